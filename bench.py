@@ -54,7 +54,7 @@ def _peaks():
 _KERNEL_SRC = {"gemm_mxf4_kernel": "gemm_mxf4.cu", "gemm_mxf4_pair_kernel": "gemm_mxf4_pair.cu",
                "act_quant8_kernel": "quant_mxfp8.cu", "act_quant_rfq8_amax_kernel": "quant_mxfp8.cu",
                "act_quant_rfq8_kernel": "quant_mxfp8.cu",
-               "gemm_mxf4_fused_kernel": "gemm_mxf4_fused.cu",
+               "gemm_small_kernel": "gemm_small.cu",
                "act_quant_mxfp4_kernel": "quant_mxfp4.cu", "act_quant_mxfp4_amax_kernel": "quant_mxfp4.cu",
                "gemm_hif4_kernel": "gemm_hif4.cu", "act_quant_hif4_kernel": "quant_hif4.cu",
                "act_quant_hif4_amax_kernel": "quant_hif4.cu"}
@@ -110,7 +110,7 @@ def _src_hash(kernel: str):
     d = os.path.join(HERE, "paper_2608_26581_gb300", "csrc")
     m = hashlib.sha256()
     extra = ("mxfp4_math.cuh",) if kernel in ("act_quant_mxfp4_kernel", "act_quant_mxfp4_amax_kernel",
-                                              "gemm_mxf4_fused_kernel", "act_quant8_kernel", "act_quant_rfq8_kernel",
+                                              "gemm_small_kernel", "act_quant8_kernel", "act_quant_rfq8_kernel",
                                               "act_quant_rfq8_amax_kernel", "gemm_mxf4_pair_kernel") else ()
     for n in (_KERNEL_SRC[kernel], "ptx.cuh", "internal.h") + extra:
         m.update(open(os.path.join(d, n), "rb").read())
@@ -759,11 +759,12 @@ def run_rfq(args):
         t_peak, t_peak_sust = pk["bf16_burst"] * FP4_OVER_BF16, pk["bf16_sust"] * FP4_OVER_BF16
         t_src = (f"{pk['src']} bf16 burst {pk['bf16_burst']} TFLOP/s x {FP4_OVER_BF16:g} "
                  f"(nominal dense FP4/BF16 ratio), of {pk['src']}")
-        # CTA pairs beyond one 128-row tile; grouped launches whose groups
+        # CTA pairs beyond one 128-row tile (the workloads of few rows may take
+        # gemm_small_kernel instead: the library chooses by estimated time); grouped launches whose groups
         # average under 2048 stacked rows run 128-row tiles on single CTAs
         grouped_single = grouped and Mb < 2048 * spec.groups
         # (fused: CTA pairs with the quantizer in their epilogue warps beyond 128 rows)
-        t_kernel = ("gemm_mxf4_pair_kernel" if M > 128 else "gemm_mxf4_fused_kernel") if fused else (
+        t_kernel = ("gemm_mxf4_pair_kernel" if M > 128 else "gemm_small_kernel") if fused else (
             "gemm_mxf4_kernel" if M <= 128 or grouped_single else "gemm_mxf4_pair_kernel")
     if hif4:
         aq_bytes = _act_quant_bytes(Mb, K, "hif4", not no_res, operand=not quant_only)

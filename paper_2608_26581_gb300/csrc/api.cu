@@ -434,6 +434,16 @@ extern "C" {
 rfq_status rfq_linear(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
                       const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, void *stream)
 {
+    return linear_rows(xq, xr, phi, phi_r_s, wq, y, out_dtype, workspace, stream, xq ? xq->rows : 0);
+}
+
+} // extern "C"
+
+namespace rfq {
+rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
+                       const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, void *stream,
+                       int64_t plan_rows)
+{
     bool launch = false;
     const rfq_status s = linear_check(xq, xr, phi, phi_r_s, wq, y, out_dtype, workspace, &launch, true);
     if (s != RFQ_OK || !launch)
@@ -478,10 +488,10 @@ rfq_status rfq_linear(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_
     a.status = static_cast<int32_t *>(workspace);
     a.f8 = f8;
     a.w4 = f8 && wq->fmt == RFQ_FMT_MXFP4;
+    a.plan_rows = plan_rows;
     return gemm_done(launch_gemm_mxf4(a, st), workspace, st);
 }
-
-} // extern "C"
+} // namespace rfq
 
 namespace {
 // Workspace of rfq_linear_fused.  M <= 128 (the single-CTA fused kernel):
@@ -585,19 +595,20 @@ rfq_status rfq_linear_fused(const void *x_bf16, int64_t M, int64_t K, const rfq_
         return gemm_done(launch_gemm_mxf4_pair(a, static_cast<cudaStream_t>(stream)), workspace,
                          static_cast<cudaStream_t>(stream));
     }
-    GemmFusedArgs a;
+    GemmSmallArgs a = {};
     a.x = x_bf16;
-    a.b_codes = wq->codes;
-    a.b_sf = wq->scales;
+    a.w = wq->codes;
+    a.w_sf = wq->scales;
     a.y = y;
     a.out_bf16 = out_dtype == RFQ_OUT_BF16;
     a.residual = mode == RFQ_FALLBACK_ALL;
+    a.fused = 1;
     a.M = M;
     a.N = N;
     a.K = K;
     a.status = static_cast<int32_t *>(workspace);
-    return gemm_done(launch_gemm_mxf4_fused(a, static_cast<cudaStream_t>(stream)), workspace,
-                         static_cast<cudaStream_t>(stream));
+    return gemm_done(launch_gemm_small(a, M, static_cast<cudaStream_t>(stream)), workspace,
+                     static_cast<cudaStream_t>(stream));
 }
 
 rfq_status rfq_linear_mixed(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,

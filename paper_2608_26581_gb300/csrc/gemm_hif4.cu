@@ -585,6 +585,24 @@ cudaError_t launch_conv(const GemmHif4Args &a, cudaStream_t st)
 
 cudaError_t launch_gemm_hif4(const GemmHif4Args &a, cudaStream_t st)
 {
+    if (a.a_bf16) {
+        // as for the MXFP4 GEMM: 32 x 12288 x 4096 takes 22 us there against
+        // 111 us here; 4096 rows stay here
+        GemmSmallArgs s = {};
+        s.x = a.a_codes;
+        s.r = a.r_codes;
+        s.w = a.b_bf16;
+        s.y = a.y;
+        s.out_bf16 = a.out_bf16;
+        s.residual = a.r_codes != nullptr;
+        s.bf16 = 1;
+        s.M = a.M;
+        s.N = a.N;
+        s.K = a.K;
+        s.status = a.status;
+        if (gemm_small_takes(s, a.M))
+            return launch_gemm_small(s, a.M, st);
+    }
     return a.a_bf16 ? launch_conv<false>(a, st) : launch_conv<true>(a, st);
 }
 

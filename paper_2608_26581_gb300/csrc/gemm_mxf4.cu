@@ -739,6 +739,29 @@ cudaError_t launch_gemm_mxf4(const GemmMxf4Args &a, cudaStream_t st)
     // than the pair saves (Qwen3-VL-30B experts, ~320 rows each: 0.106 ms
     // here against 0.112 ms on pairs).
     const bool grp = a.groups > 0;
+    if (!grp && !a.f8) {
+        // Few rows, or few output tiles: the cluster-split kernel where its
+        // estimated time is the smaller (choose() in gemm_small.cu).  48 x 12288
+        // x 4096: 10.3 us there against 34 us here (16 tiles for 152 SMs); 128 x
+        // 5120 x 24576: 22.6 against 21.9 us (96 tiles), which stays here.
+        GemmSmallArgs s = {};
+        s.x = a.a_codes;
+        s.r = a.r_codes;
+        s.w = a.b_codes;
+        s.x_sf = a.a_sf;
+        s.r_sf = a.r_sf;
+        s.w_sf = a.b_sf;
+        s.y = a.y;
+        s.out_bf16 = a.out_bf16;
+        s.residual = a.r_codes != nullptr;
+        s.M = a.M;
+        s.N = a.N;
+        s.K = a.K;
+        s.status = a.status;
+        const int64_t rows = a.plan_rows ? a.plan_rows : a.M;
+        if (gemm_small_takes(s, rows))
+            return launch_gemm_small(s, rows, st);
+    }
     const bool grp_single = grp && !a.f8 && a.M < (int64_t)2048 * a.groups;
     if ((a.M > BM && !grp_single) || a.f8 || (grp && !grp_single))
         return launch_gemm_mxf4_pair(a, st);

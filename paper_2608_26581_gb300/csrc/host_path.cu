@@ -144,7 +144,7 @@ rfq_status rfq_linear_host(const void *x_host, int64_t M, int64_t K, const rfq_f
         if ((s = rfq_quantize_act(static_cast<uint8_t *>(x_dev) + xoff, m, K, fb, &q, xr ? &r : nullptr, ph,
                                   stream)) != RFQ_OK)
             return s;
-        if ((s = rfq_linear(&q, xr ? &r : nullptr, ph, r_s, wq, yd, out_dtype, workspace, stream)) != RFQ_OK)
+        if ((s = linear_rows(&q, xr ? &r : nullptr, ph, r_s, wq, yd, out_dtype, workspace, stream, M)) != RFQ_OK)
             return s;
         const size_t yoff = (size_t)r0 * (size_t)N * ybytes, ylen = (size_t)m * (size_t)N * ybytes;
         if (cudaEventRecord(y_ready, st) != cudaSuccess || cudaStreamWaitEvent(cs.d2h, y_ready, 0) != cudaSuccess ||

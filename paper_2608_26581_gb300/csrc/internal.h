@@ -122,6 +122,7 @@ struct GemmMxf4Args {
     void *y;
     int out_bf16;
     int64_t M, N, K;
+    int64_t plan_rows = 0;                     // rows of the whole matrix when M is a chunk of it (0: M)
     int32_t *status;
     int f8 = 0;                                // every operand MXFP8 (E4M3): kind::mxf8f6f4, CTA pairs
     int w4 = 0;                                // with f8: W~ MXFP4 [N][K/2] (32-byte aligned), multiplied
@@ -148,17 +149,23 @@ cudaError_t launch_gemm_mxf4(const GemmMxf4Args &a, cudaStream_t st);
 // CTA-pair kernel (gemm_mxf4_pair.cu), used by launch_gemm_mxf4 when M > 128.
 cudaError_t launch_gemm_mxf4_pair(const GemmMxf4Args &a, cudaStream_t st);
 
-// ---- RFQ linear with the quantizer fused into the GEMM (gemm_mxf4_fused.cu)
-struct GemmFusedArgs {
-    const void *x;                 // bf16 [M][K]
-    const void *b_codes, *b_sf;    // MXFP4 weight, MMA-layout scales
+// ---- RFQ GEMM for few rows (gemm_small.cu): X (or its bf16 values) as the
+// narrow MMA side, the reduction split over a cluster.  MXFP4 operands with
+// MMA-layout scales; bf16 = 1: exact bf16 expansions (HiF4), no scales;
+// fused = 1: x is bf16 X, quantized inside the kernel (M <= 128).
+struct GemmSmallArgs {
+    const void *x, *r, *w;         // r unused without a residual or with fused
+    const void *x_sf, *r_sf, *w_sf;
     void *y;
-    int out_bf16;
-    int residual;                  // 1: phi = 1 everywhere, 0: plain W4A4
+    int out_bf16, residual, bf16, fused;
     int64_t M, N, K;
     int32_t *status;
 };
-cudaError_t launch_gemm_mxf4_fused(const GemmFusedArgs &a, cudaStream_t st);
+// Whether this kernel is the faster one for a layer of plan_rows rows (the
+// rows of the whole matrix when a caller passes it in chunks: every chunk
+// then sums in the same order), and its launch.
+bool gemm_small_takes(const GemmSmallArgs &a, int64_t plan_rows);
+cudaError_t launch_gemm_small(const GemmSmallArgs &a, int64_t plan_rows, cudaStream_t st);
 
 // ---- HiF4 quantization (quant_hif4.cu); metadata layout RFQ_SCALE_MMA is
 // block-major [K/64][rows rounded up to 128]
@@ -211,6 +218,13 @@ cudaError_t launch_fp4_mma_peak(int pair, int64_t iters, int32_t *status, double
 rfq_status linear_check(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
                         const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, bool *launch,
                         bool check_ws);
+
+// rfq_linear on some rows of a matrix of plan_rows rows: the kernel and its
+// reduction split are those of the whole matrix, so every chunk's outputs are
+// summed in the whole's order.
+rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
+                       const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, void *stream,
+                       int64_t plan_rows);
 
 // Blocks of `threads` threads (and `smem` dynamic shared bytes) of `kern`
 // resident on one SM at once (cached per kernel): grid-stride kernels launch

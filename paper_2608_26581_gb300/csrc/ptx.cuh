@@ -20,6 +20,21 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
     return t;
 }
 
+// True in exactly one lane of a converged warp.  The compiler knows that at
+// most one lane passes, and so issues the tensor-core and TMA instructions
+// under it straight from uniform registers; under a plain `lane == 0` it
+// cannot tell, and each tcgen05.mma took 67 cycles to issue instead of the
+// 39 that the narrowest MMA itself takes (128 x 16).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "elect.sync _|p, 0xffffffff;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(p));
+    return p != 0;
+}
+
 // ---------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
@@ -91,7 +106,12 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
 // most `limit_ns` nanoseconds of wall time, or until `*abort_word` (a status
 // word in global memory, may be null) becomes non-zero.  Returns false on
 // timeout or abort.  CLUSTER selects cluster-scope acquire.
-template <bool CLUSTER = false>
+// LATE_CLOCK first reads the clock after 64 tests, so that a wait that is
+// nearly over, the usual one, does not pay for reading it: for kernels whose
+// stages are short (without it the few-rows GEMM takes 0.33 us per stage
+// instead of 0.29; with it the mixed-rate GEMM's many waiting warps poll so
+// much that it takes 4% longer).
+template <bool CLUSTER = false, bool LATE_CLOCK = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64_t limit_ns,
                                           const volatile int32_t *abort_word = nullptr)
 {
@@ -99,12 +119,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64
     auto test = [&]() { return CLUSTER ? mbar_try_wait_cluster(a, parity) : mbar_try_wait(a, parity); };
     if (test())
         return true;
-    const uint64_t t0 = globaltimer_ns();
+    uint64_t t0 = LATE_CLOCK ? 0 : globaltimer_ns();
     for (uint32_t i = 1;; ++i) {
         if (test())
             return true;
         if ((i & 63) == 0) {
-            if (globaltimer_ns() - t0 > limit_ns)
+            const uint64_t t = globaltimer_ns();
+            if (LATE_CLOCK && t0 == 0)
+                t0 = t;
+            if (t - t0 > limit_ns)
                 return false;
             if (abort_word && *abort_word != 0)
                 return false;
@@ -389,6 +412,28 @@ __device__ __forceinline__ void tmem_st_32x32b_x4(uint32_t taddr, uint32_t r0, u
 {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(r0), "r"(r1),
                  "r"(r2), "r"(r3)
+                 : "memory");
+}
+
+// The same with 16 and 32 columns.
+__device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_t *r)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+                 "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+                 : "memory");
+}
+
+__device__ __forceinline__ void tmem_st_32x32b_x32(uint32_t taddr, const uint32_t *r)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+                 "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+                 "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+                 "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
+                 "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
+                 "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
                  : "memory");
 }
 
