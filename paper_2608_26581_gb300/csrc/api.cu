@@ -434,7 +434,7 @@ extern "C" {
 rfq_status rfq_linear(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
                       const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, void *stream)
 {
-    return linear_rows(xq, xr, phi, phi_r_s, wq, y, out_dtype, workspace, stream, xq ? xq->rows : 0);
+    return linear_rows(xq, xr, phi, phi_r_s, wq, y, out_dtype, workspace, stream, 0);
 }
 
 } // extern "C"

@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
     const volatile int32_t *gstat = status;
 
     if (threadIdx.x == 0) {
+        grid_dependency_wait();
         S.abort_flag = *gstat;
         S.wait_ns = ws_wait_limit_ns(status);
     }
@@ -538,9 +539,9 @@ cudaError_t launch_variant(const CUtensorMap &ta, const CUtensorMap &tr, const C
     const int grid = (int)(tiles < num_sms() ? tiles : num_sms());
     const int phi_blocks = a.phi_r_s / BK;
     const int phi_cols = a.phi ? (int)((a.K + a.phi_r_s - 1) / a.phi_r_s) : 0;
-    kern<<<grid, PHI ? THREADS + 32 : THREADS, smem, st>>>(ta, tr, tb, ty, (const uint32_t *)a.a_meta, (const uint32_t *)a.r_meta, a.phi,
-                                      phi_blocks, phi_cols, a.y, (int)a.M, (int)a.N, (int)a.K, a.status);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(grid), PHI ? THREADS + 32 : THREADS, smem, st, true, ta, tr, tb, ty,
+                            (const uint32_t *)a.a_meta, (const uint32_t *)a.r_meta, a.phi, phi_blocks, phi_cols, a.y,
+                            (int)a.M, (int)a.N, (int)a.K, a.status);
 }
 
 template <bool CONV>

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
 
     // A bounded wait of an earlier CTA or call gave up: do nothing.
     if (threadIdx.x == 0) {
+        grid_dependency_wait();
         S.abort_flag = *gstat;
         S.wait_ns = ws_wait_limit_ns(status);
     }
@@ -721,10 +722,9 @@ cudaError_t launch_variant(const CUtensorMap &ta, const CUtensorMap &tr, const C
     const int grid = (int)(tiles < num_sms() ? tiles : num_sms());
     const int phi_chunks = a.phi_r_s / 128;
     const int phi_cols = a.phi ? (int)((a.K + a.phi_r_s - 1) / a.phi_r_s) : 0;
-    kern<<<grid, PHI ? THREADS + 32 : THREADS, kSmemBytes, st>>>(
-        ta, tr, tb, ty, (const uint8_t *)a.a_sf, (const uint8_t *)a.r_sf, (const uint8_t *)a.b_sf, a.phi, phi_chunks,
-        phi_cols, (int)a.M, (int)a.N, (int)a.K, a.status, a.group_off, a.groups, a.y);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(grid), PHI ? THREADS + 32 : THREADS, kSmemBytes, st, a.plan_rows == 0, ta, tr,
+                            tb, ty, (const uint8_t *)a.a_sf, (const uint8_t *)a.r_sf, (const uint8_t *)a.b_sf, a.phi,
+                            phi_chunks, phi_cols, (int)a.M, (int)a.N, (int)a.K, a.status, a.group_off, a.groups, a.y);
 }
 
 } // namespace

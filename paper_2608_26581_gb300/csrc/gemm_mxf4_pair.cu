@@ -264,6 +264,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
         }
         // A bounded wait of an earlier CTA or call gave up: skip the work
         // (both CTAs still meet at the cluster barriers).
+        grid_dependency_wait();
         S.abort_flag = *gstat;
         S.wait_ns = ws_wait_limit_ns(status);
         fence_mbar_init();
@@ -289,6 +290,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
         // computes nothing.  The prefix of 256-row pairs maps a tile index to
         // its group.
         int bad = 0;
+        grid_dependency_wait();
         if (G > 0) {
             for (int e = lane; e <= G; e += 32)
                 S.grp_off[e] = __ldg(group_off + e);
@@ -1132,10 +1134,10 @@ cudaError_t launch_variant(const CUtensorMap &ta, const CUtensorMap &tr, const C
         fq.ctr = a.fq_ctr;
         fq.ring = a.fq_ring;
     }
-    kern<<<grid, PHI ? THREADS + 32 : THREADS, kSmemBytes, st>>>(
-        ta, tr, tb, ty, tb4 ? *tb4 : tb, (const uint8_t *)a.a_sf, (const uint8_t *)a.r_sf, (const uint8_t *)a.b_sf, a.phi, phi_chunks,
-        phi_cols, (int)a.M, (int)a.N, (int)a.K, a.status, a.group_off, a.groups, a.y, fq);
-    return cudaGetLastError();
+    return launch_dependent(kern, dim3(grid), PHI ? THREADS + 32 : THREADS, kSmemBytes, st, a.plan_rows == 0, ta, tr,
+                            tb, ty, tb4 ? *tb4 : tb, (const uint8_t *)a.a_sf, (const uint8_t *)a.r_sf,
+                            (const uint8_t *)a.b_sf, a.phi, phi_chunks, phi_cols, (int)a.M, (int)a.N, (int)a.K,
+                            a.status, a.group_off, a.groups, a.y, fq);
 }
 
 } // namespace

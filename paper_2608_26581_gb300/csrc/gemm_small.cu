@@ -120,6 +120,7 @@ struct Shape {
     int x_atoms;        // 128-row scale atoms a tile's rows of X can span (1 or 2)
     int tmem_cols, acc_cols;    // allocated columns; columns between the accumulators of two W~ blocks
     int sf_col0;                // first scale slot's column
+    int prefetch;               // k-stages of W~ prefetched into L2 at the start
     int res, cat, out_bf16;
 };
 
@@ -200,10 +201,22 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
     if (threadIdx.x == 32 * SFP_WARP) {
         // the workspace's words in one load (they are read before anything is
         // copied: one trip to L2 instead of three)
+        grid_dependency_wait();
         const int4 w = __ldcv(reinterpret_cast<const int4 *>(status));
         S.abort_flag = w.x;              // a bounded wait of an earlier CTA or call gave up: compute nothing
         S.wait_ns = w.y > 0 ? (uint64_t)w.y * 1000ull : kWaitLimitNs;
         S.hold = w.z;
+    }
+    if (warp == 0) {
+        // Before the kernel ahead of this one has ended (see the launch), W~
+        // starts on its way from HBM to L2: the first PREFETCH stages' tiles, a
+        // hint that is right whatever that kernel writes.
+        if (elect_one())
+            for (int p = 0; p < min(n_st, sh.prefetch); ++p) {
+                tma_prefetch_2d(&tmW, (k_lo + p) * ROW, n0);
+                if (!SWAP && WT > 1 && nw > 1)
+                    tma_prefetch_2d(&tmW, (k_lo + p) * ROW, n0 + WROWS);
+            }
     }
     if (warp == 2 && lane == 0) {
         prefetch_tmap(&tmW);
@@ -753,6 +766,10 @@ bool make_shape(const GemmSmallArgs &a, int64_t plan_rows, const Plan &p, Shape 
         st = st < slots ? st : slots;
     }
     s.stages = st;
+    // (of 0, 4, 16 and 64 stages in a layer call: 1 x 4096 x 24576 15.5 / 15.0 /
+    // 15.9 / 15.9 us, HiF4 32 x 12288 x 4096 27.0 / 26.4 / 25.6 / 28.5, 333 rows best
+    // with none; the fused form has no quantizer ahead of it)
+    s.prefetch = plan_rows > 128 || a.fused ? 0 : f4 ? 4 : 16;
     const int ps = swap ? 2 * WROWS + 4 : s.NT;
     if (a.fused && (swap || a.M > 128))
         return false;
@@ -784,13 +801,17 @@ cudaError_t launch_variant(const GemmSmallArgs &a, const Plan &p, const Shape &s
     cfg.blockDim = dim3(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * CONV_WARP0);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)p.cs;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    // The kernel ahead in the stream is usually the activation quantizer (2-4 us
+    // for few rows): this one's set-up and its first look at W~ overlap it.
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, kern, tw, tx, tr, (const uint8_t *)a.w_sf, (const uint8_t *)a.x_sf,
                               (const uint8_t *)a.r_sf, FUSED ? (const uint4 *)a.x : nullptr, a.y, a.status, s);
 }

@@ -122,7 +122,8 @@ struct GemmMxf4Args {
     void *y;
     int out_bf16;
     int64_t M, N, K;
-    int64_t plan_rows = 0;                     // rows of the whole matrix when M is a chunk of it (0: M)
+    int64_t plan_rows = 0;                     // rows of the whole matrix when M is a chunk of it in a call
+                                               // from host memory (0: a device call on M rows)
     int32_t *status;
     int f8 = 0;                                // every operand MXFP8 (E4M3): kind::mxf8f6f4, CTA pairs
     int w4 = 0;                                // with f8: W~ MXFP4 [N][K/2] (32-byte aligned), multiplied
@@ -219,9 +220,9 @@ rfq_status linear_check(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint
                         const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, bool *launch,
                         bool check_ws);
 
-// rfq_linear on some rows of a matrix of plan_rows rows: the kernel and its
-// reduction split are those of the whole matrix, so every chunk's outputs are
-// summed in the whole's order.
+// rfq_linear on some rows of a matrix of plan_rows rows (0: on the whole one):
+// the kernel and its reduction split are those of the whole matrix, so every
+// chunk's outputs are summed in the whole's order.
 rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
                        const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, void *stream,
                        int64_t plan_rows);
@@ -230,6 +231,27 @@ rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8
 // resident on one SM at once (cached per kernel): grid-stride kernels launch
 // at most that many per SM, so no partial second wave trails the first.
 int resident_blocks_per_sm(const void *kern, int threads, size_t smem);
+
+// Launch of a GEMM kernel that calls grid_dependency_wait before its first
+// read of global memory: with `dependent` its set-up may overlap the end of
+// the kernel ahead of it in the stream (the activation quantizer: 1.0-1.7 us
+// less per layer).  Calls from host memory (rfq_linear_host) launch plainly.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                    bool dependent, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // Number of SMs of the current device (cached).
 int num_sms();

@@ -153,6 +153,23 @@ __device__ __forceinline__ bool held_start_wait(const int32_t *ws, uint64_t limi
     }
 }
 
+// ---------------------------------------------------------------- dependent launches
+
+// Lets the next kernel of the stream, if it was launched to allow it, start
+// its set-up while this grid still runs (it waits in grid_dependency_wait for
+// this grid's end and its memory).  No effect on any other kernel.
+__device__ __forceinline__ void grid_launch_dependents()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Waits until the grids this one depends on have ended and their memory is
+// visible (at once when the launch was an ordinary one).
+__device__ __forceinline__ void grid_dependency_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- clusters
 
 __device__ __forceinline__ uint32_t cluster_ctarank()
@@ -214,6 +231,15 @@ __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *m
         " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
         "l"(reinterpret_cast<uint64_t>(m)), "r"(cbar), "r"(x), "r"(y)
         : "memory");
+}
+
+// Brings the tile a tma_load_2d would copy into L2: a hint, nothing reads it.
+__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *m, int32_t x, int32_t y)
+{
+    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
+                     reinterpret_cast<uint64_t>(m)),
+                 "r"(x), "r"(y)
+                 : "memory");
 }
 
 // Contiguous bulk copy global -> shared (16-byte aligned, size % 16 == 0).

@@ -19,6 +19,7 @@
 
 #include "internal.h"
 #include "mxfp4_math.cuh"
+#include "ptx.cuh"
 
 namespace rfq {
 namespace {
@@ -57,6 +58,7 @@ __global__ void __launch_bounds__(256) act_quant_mxfp4_kernel(const uint4 *__res
                                                              const uint8_t *__restrict__ phi, int p_s, int r_s,
                                                              int64_t pad_rows)
 {
+    grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
     const int lane = threadIdx.x & 31;
     const int kblocks = (int)(K >> 5);
     const int segs = (kblocks + 31) / 32;
@@ -202,6 +204,7 @@ __global__ void __launch_bounds__(256, 3)
                                 uint8_t *__restrict__ mscales, uint32_t *__restrict__ rcodes,
                                 uint8_t *__restrict__ rscales, uint8_t *__restrict__ phi, float tau)
 {
+    grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
     constexpr int R = kAmaxRows;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t kchunks = K >> 3;
