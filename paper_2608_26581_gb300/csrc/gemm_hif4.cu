@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             int p = 0, it = 0;
             bool stop = false;
             if (!held_start_wait(status, wl)) { // a test-held start never opened
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             int p = 0, it = 0;
             bool stop = false;
             const uint32_t idesc = idesc_bf16(BM, BN);

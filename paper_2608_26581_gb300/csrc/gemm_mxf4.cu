@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {   // (not `lane == 0`: see elect_one)
             int p = 0, it = 0; // p: stages issued so far (ring position)
             bool stop = false;
             if (!held_start_wait(status, wl)) { // a test-held start never opened
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {   // (not `lane == 0`: see elect_one)
             int p = 0, it = 0;
             bool stop = false;
             for (int tile = blockIdx.x; tile < tiles && !stop; tile += gridDim.x, ++it) {

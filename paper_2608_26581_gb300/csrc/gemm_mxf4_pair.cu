@@ -7,20 +7,21 @@
 // k-stage an SM streams 52 KB (codes and scale atoms) for 1,024 cycles of MMA
 // work, 24% less than the 68 KB of a single-CTA 128 x 256 tile.
 //
-// Per CTA (448 threads, 480 with selective phi; one CTA per SM):
+// Per CTA (480 threads, 512 with selective phi; one CTA per SM):
 //   warp 0      TMA producer.  The codes (own A and R rows, own W~ half) are
 //               CTA-pair copies that complete on the EVEN CTA's stage
 //               barrier, which the even CTA's producer arms with the bytes of
-//               both CTAs; the scale atoms (own A / R rows, both 128-row W~
-//               atoms of the tile) are bulk copies into this CTA's shared
-//               memory, on its own barrier.
+//               both CTAs.
 //   warp 1      even CTA: MMA issuer (main + residual MMA per K=64 step,
 //               same W~ descriptor, same accumulator: Sec. 4.3)
 //   warps 2-9   epilogue: TMEM -> registers -> bf16 / fp32 -> shared-memory
 //               staging -> TMA stores of this CTA's 128 rows
 //   warps 10-13 scale writers: this CTA's scale words from shared memory into
 //               its TMEM with tcgen05.st, one warp per TMEM lane quarter
-//   warp 14     (selective phi only) phi reader: one record per output tile
+//   warp 14     scale producer: the scale atoms (own A / R rows, both 128-row
+//               W~ atoms of the tile), bulk copies into this CTA's shared
+//               memory, on its own barrier
+//   warp 15     (selective phi only) phi reader: one record per output tile
 //               of this CTA (double-buffered) with a bit per k-stage, set
 //               when the stage needs its residual, and their count
 // TMEM (512 columns per CTA): a 256-column accumulator (this CTA's 128 rows
@@ -85,8 +86,9 @@ constexpr int SF_SLOT_COLS = 32;         // A chunk c at 4c, R at 8 + 4c, W~ at 
 constexpr int SF_SLOTS = 4;
 constexpr int EPI_WARPS = 8;
 constexpr int SF_WARPS = 4;
-constexpr int THREADS = 64 + 32 * (EPI_WARPS + SF_WARPS);
-constexpr int PHI_WARP = THREADS / 32;   // the phi reader: one warp beyond THREADS
+constexpr int SFP_WARP = 2 + EPI_WARPS + SF_WARPS;   // the scale-atom producer
+constexpr int THREADS = 32 * (SFP_WARP + 1);
+// (with selective phi one warp more: the phi reader)
 constexpr int REC_WORDS = 64;            // phi record: up to 2048 full k-stages (K <= 524288)
 constexpr int GRP_MAX = 128;             // groups of the grouped GEMM
 constexpr int YSTAGE = 2048;             // per epilogue warp: 32 rows x 64 bytes of Y
@@ -260,7 +262,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
         mbar_init(&S.drain, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&S.phi_full[i], 32);
-            mbar_init(&S.phi_empty[i], 1);
+            mbar_init(&S.phi_empty[i], 2);   // (both producers)
         }
         // A bounded wait of an earlier CTA or call gave up: skip the work
         // (both CTAs still meet at the cluster barriers).
@@ -360,13 +362,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
         return c;
     };
 
-    if (warp == 0) {
-        // ------------------------------------------------ TMA producer (both CTAs)
-        if (lane == 0 && !skip) {
+    // TMA producers (both CTAs): warp 0 copies a stage's codes (OPS), warp
+    // SFP_WARP its scale atoms, in the same order.  A copy takes the issuing
+    // lane 80-100 cycles, so one producer needed most of a stage's MMA time
+    // for its seven or eight (the mixed-rate form more than all of it).  Layer
+    // times with one producer and with two: mixed rate 8190 x 5120 x 13824 500
+    // and 489 us, MXFP4 4096 x 4096 x 24576 226 and 222 (the single-CTA kernel,
+    // whose stages take longer, gained nothing and keeps one).
+    auto producer = [&](auto ops_t) {
+        constexpr bool OPS = decltype(ops_t)::value;
+        if (!skip && elect_one()) {
             const uint32_t full0 = mapa_shared(smem_u32(&S.full[0]), 0);   // the even CTA's barriers
             int p = 0, it = 0;
             bool stop = false;
-            int fq_tile_ok = -1;   // FQ: a 128-row tile whose every unit is quantized
+            [[maybe_unused]] int fq_tile_ok = -1;   // FQ: a 128-row tile whose every unit is quantized
             if (!held_start_wait(status, wl)) { // a test-held start never opened
                 flag_timeout(S, status);
                 stop = true;
@@ -419,18 +428,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
                             fence_proxy_async_global();
                         }
                     }
-                    const int c0 = CPS * ks, cx = c0 * (F8 ? 128 : 64); // first chunk, its byte column
+                    const int c0 = CPS * ks;                            // first chunk
+                    [[maybe_unused]] const int cx = c0 * (F8 ? 128 : 64);   // its byte column
                     if (PHI)
-                        S.stage_info[slot] = info;
+                        S.stage_info[slot] = info;   // (both producers: whichever barrier a reader waits for)
                     Stage &st = S.st[slot];
-                    const uint32_t bar = full0 + 8 * slot;
-                    const uint32_t sfbytes = (uint32_t)nch * ATOM;
-                    uint64_t *sbar = &S.sf_full[slot];
-                    if (F8 == F8_MIXED) {
+                    if constexpr (!OPS) {
+                        const uint32_t sfbytes = (uint32_t)nch * ATOM;
+                        uint64_t *sbar = &S.sf_full[slot];
+                        mbar_arrive_expect_tx(sbar, nb * sfbytes + (rows_in ? (res_on ? 2 : 1) * sfbytes : 0));
+                        if (rows_in) {
+                            bulk_load(st.sfa, sfa + ((int64_t)sf_tile * kc + c0) * ATOM, sfbytes, sbar);
+                            if (res_on)
+                                bulk_load(st.sfr, sfr + ((int64_t)sf_tile * kc + c0) * ATOM, sfbytes, sbar);
+                        }
+                        for (int h = 0; h < nb; ++h)
+                            bulk_load(st.sfb + h * 2 * ATOM, sfb + ((int64_t)(atom0 + h) * kc + c0) * ATOM, sfbytes,
+                                      sbar);
+                    } else if constexpr (F8 == F8_MIXED) {
                         // X~ and W~ packed (64-byte rows) side by side in the A tile;
                         // with a residual, X^ as E4M3 in the R tile.  The W~ half lands
                         // on this CTA's own barrier: its scale writers expand it into
                         // the B tile in the padded 4-bit form the residual MMAs read
+                        const uint32_t bar = full0 + 8 * slot;
                         if (lead)
                             mbar_arrive_expect_tx(&S.full[slot], 2 * (A_BYTES / 2 + (res_on ? A_BYTES : 0)));
                         tma_load_2d_pair(st.a, &tmA, bar, c0 * 64, a_y);
@@ -440,6 +460,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
                         if (res_on)
                             tma_load_2d_pair(st.r, &tmR, bar, cx, a_y);
                     } else {
+                        const uint32_t bar = full0 + 8 * slot;
                         if (lead)
                             mbar_arrive_expect_tx(&S.full[slot], 2 * (A_BYTES + B_TX + (res_on ? A_BYTES : 0)));
                         tma_load_2d_pair(st.a, &tmA, bar, cx, a_y);
@@ -447,15 +468,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
                             tma_load_2d_pair(st.r, &tmR, bar, cx, a_y);
                         tma_load_2d_pair(st.b, &tmB, bar, cx, tc.w_row0 + (int)rank * BN_HALF);
                     }
-                    mbar_arrive_expect_tx(sbar, nb * sfbytes + (rows_in ? (res_on ? 2 : 1) * sfbytes : 0));
-                    if (rows_in) {
-                        bulk_load(st.sfa, sfa + ((int64_t)sf_tile * kc + c0) * ATOM, sfbytes, sbar);
-                        if (res_on)
-                            bulk_load(st.sfr, sfr + ((int64_t)sf_tile * kc + c0) * ATOM, sfbytes, sbar);
-                    }
-                    for (int h = 0; h < nb; ++h)
-                        bulk_load(st.sfb + h * 2 * ATOM, sfb + ((int64_t)(atom0 + h) * kc + c0) * ATOM, sfbytes,
-                                  sbar);
                     ++p;
                 };
                 if constexpr (!PHI) {
@@ -502,17 +514,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
             }
             if (stop || S.abort_flag)
                 // wait (bounded) until the copies of the last stages landed: this
-                // CTA's scale atoms, and (even CTA) both CTAs' codes
+                // CTA's scale atoms, or (even CTA) both CTAs' codes
                 for (int q = max(0, p - STAGES); q < p; ++q) {
-                    (void)mbar_wait(&S.sf_full[q % STAGES], (q / STAGES) & 1, wl);
+                    if (!OPS) {
+                        (void)mbar_wait(&S.sf_full[q % STAGES], (q / STAGES) & 1, wl);
+                        continue;
+                    }
                     if (F8 == F8_MIXED)
                         (void)mbar_wait(&S.w4_full[q % STAGES], (q / STAGES) & 1, wl);
                     if (lead)
                         (void)mbar_wait(&S.full[q % STAGES], (q / STAGES) & 1, wl);
                 }
         }
+    };
+    if (warp == 0) {
+        producer(Bool<true>{});
+    } else if (warp == SFP_WARP) {
+        producer(Bool<false>{});
     } else if (warp == 1) {
-        if (lane == 0 && !skip && lead) {
+        if (!skip && lead && elect_one()) {
             // -------------------------------------------- MMA issuer (even CTA)
             int p = 0, it = 0;
             bool stop = false;
@@ -910,7 +930,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
         }
         if (lane == 0)
             bulk_wait_group<0>(); // every TMA store of this warp has completed
-    } else if (warp < PHI_WARP) {
+    } else if (warp < SFP_WARP) {
         // ------------------------------------------------ scale writers (warps 10..13)
         // Warp quarter q writes TMEM lanes 32q..32q+31; every quarter holds
         // the same words: column j of lane i carries the four scales of row
@@ -1027,7 +1047,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
             }
         }
     } else if (PHI) {
-        // ------------------------------------------------ phi reader (warp 14)
+        // ------------------------------------------------ phi reader (warp 15)
         // Record of the CTA's j-th tile: chunk c of the pair's row tile m
         // (128 rows) needs its residual when phi[m][c / phi_chunks] is non-zero.
         const int my_tiles = pair < tiles ? (tiles - pair + pairs - 1) / pairs : 0;
