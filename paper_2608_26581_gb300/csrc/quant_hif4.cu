@@ -27,6 +27,7 @@
 
 #include "internal.h"
 #include "ptx.cuh"
+#include "weight_tile.cuh"
 
 namespace rfq {
 namespace {
@@ -486,8 +487,40 @@ __global__ void __launch_bounds__(512, 1) act_quant_hif4_amax_kernel(const uint4
     }
 }
 
-// One thread per (column n, 64-block) of W [K x N]: a warp reads 32
-// consecutive columns of one K row at a time.
+// The tiled weight quantizer (weight_tile.cuh) for even N.
+template <int LAYOUT>
+struct WeightHif4 {
+    static constexpr int BLK = 64, OUTB = 32, ORDER = LAYOUT == RFQ_SCALE_MMA ? WT_COLUMNS : WT_BLOCKS;
+    using Scale = uint32_t;
+    static __device__ __forceinline__ void run(const uint32_t (&raw)[64], int half, uint32_t (&code)[8], uint32_t &s)
+    {
+        float am = 0.f;
+#pragma unroll
+        for (int i = 0; i < 64; ++i)
+            am = fmaxf(am, fabsf(wt_value(raw[i], half)));
+        const int sb = am > 0.f ? hif4_scale_byte(am) : 0;
+        uint32_t bits = 0;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            float x[8], deq[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                x[i] = wt_value(raw[8 * g + i], half);
+            uint32_t gb;
+            code[g] = hif4_group(x, sb, g, gb, deq);
+            bits |= gb;
+        }
+        s = am == 0.f ? 0u : (bits | (uint32_t)sb);
+    }
+    static __device__ __forceinline__ int64_t scale_at(int64_t n, int64_t b, int64_t N, int64_t kblocks)
+    {
+        return meta_index<LAYOUT>(n, b, N, kblocks);
+    }
+    static __device__ __forceinline__ int64_t scale_count(int64_t pad_cols, int64_t kblocks) { return pad_cols * kblocks; }
+    static __device__ __forceinline__ bool in_bounds(int64_t, int64_t) { return true; }
+};
+
+// One thread per (column n, 64-block) of W [K x N]: the form for odd N.
 template <int LAYOUT>
 __global__ void __launch_bounds__(256) weight_quant_hif4_kernel(const __nv_bfloat16 *__restrict__ w, int64_t K,
                                                                int64_t N, uint8_t *__restrict__ codes,
@@ -636,6 +669,10 @@ cudaError_t launch_act_quant_hif4(const void *x, int64_t M, int64_t K, int mode,
 cudaError_t launch_weight_quant_hif4(const void *w, int64_t K, int64_t N, void *codes, void *meta, int layout,
                                      cudaStream_t st)
 {
+    if (N % 2 == 0)   // (the block-major layout's padding words are not written)
+        return layout == RFQ_SCALE_MMA
+                   ? launch_weight_tile<WeightHif4<RFQ_SCALE_MMA>>(w, K, N, N, codes, meta, st)
+                   : launch_weight_tile<WeightHif4<RFQ_SCALE_ROWMAJOR>>(w, K, N, N, codes, meta, st);
     const int64_t work = N * (K / 64);
     const unsigned blocks = (unsigned)((work + 255) / 256);
     if (layout == RFQ_SCALE_MMA)

@@ -20,6 +20,7 @@
 #include "internal.h"
 #include "mxfp4_math.cuh"
 #include "ptx.cuh"
+#include "weight_tile.cuh"
 
 namespace rfq {
 namespace {
@@ -314,8 +315,35 @@ __global__ void fill_u8_kernel(uint8_t *p, int64_t n, uint8_t v)
         p[i] = v;
 }
 
-// One thread per (column n, 32-block b) of W [K x N]: a warp reads 32
-// consecutive columns of one K row at a time (coalesced).
+// The tiled weight quantizer (weight_tile.cuh) for even N.
+template <int LAYOUT>
+struct WeightMxfp4 {
+    static constexpr int BLK = 32, OUTB = 16, ORDER = LAYOUT == RFQ_SCALE_MMA ? WT_ATOMS : WT_BLOCKS;
+    using Scale = uint8_t;
+    static __device__ __forceinline__ void run(const uint32_t (&raw)[32], int half, uint32_t (&code)[4], uint8_t &s)
+    {
+        const uint32_t am = wt_absmax2(raw);
+        const int sb = scale_byte_from_f32_bits(half ? am & 0xFFFF0000u : am << 16);
+        const float inv = pow2_neg_e(sb);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            float y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                y[i] = wt_value(raw[8 * g + i], half) * inv;
+            code[g] = e2m1x8(y);
+        }
+        s = (uint8_t)sb;
+    }
+    static __device__ __forceinline__ int64_t scale_at(int64_t n, int64_t b, int64_t, int64_t kblocks)
+    {
+        return scale_index<LAYOUT>(n, b, kblocks);
+    }
+    static __device__ __forceinline__ int64_t scale_count(int64_t pad_cols, int64_t kblocks) { return pad_cols * kblocks; }
+    static __device__ __forceinline__ bool in_bounds(int64_t i, int64_t n) { return RFQ_IN_BOUNDS(i, n); }
+};
+
+// One thread per (column n, 32-block b) of W [K x N]: the form for odd N.
 template <int LAYOUT>
 __global__ void __launch_bounds__(256) weight_quant_mxfp4_kernel(const __nv_bfloat16 *__restrict__ w, int64_t K,
                                                                 int64_t N, int64_t Npad, uint8_t *__restrict__ codes,
@@ -491,6 +519,10 @@ cudaError_t launch_weight_quant_mxfp4(const void *w, int64_t K, int64_t N, void 
                                       cudaStream_t st)
 {
     const int64_t Npad = layout == RFQ_SCALE_MMA ? ((N + 127) / 128) * 128 : N;
+    if (N % 2 == 0)
+        return layout == RFQ_SCALE_MMA
+                   ? launch_weight_tile<WeightMxfp4<RFQ_SCALE_MMA>>(w, K, N, Npad, codes, scales, st)
+                   : launch_weight_tile<WeightMxfp4<RFQ_SCALE_ROWMAJOR>>(w, K, N, Npad, codes, scales, st);
     const int64_t work = Npad * (K / 32);
     const unsigned blocks = (unsigned)((work + 255) / 256);
     if (layout == RFQ_SCALE_MMA)

@@ -18,6 +18,7 @@
 #include "internal.h"
 #include "mxfp4_math.cuh"
 #include "ptx.cuh"
+#include "weight_tile.cuh"
 
 namespace rfq {
 namespace {
@@ -384,7 +385,37 @@ __global__ void __launch_bounds__(256, 3) act_quant_rfq8_amax_kernel(const uint4
     }
 }
 
-// One thread per (column n, 32-block b) of W [K x N].
+// The tiled weight quantizer (weight_tile.cuh) for even N.
+template <int LAYOUT>
+struct WeightMxfp8 {
+    static constexpr int BLK = 32, OUTB = 32, ORDER = LAYOUT == RFQ_SCALE_MMA ? WT_ATOMS : WT_BLOCKS;
+    using Scale = uint8_t;
+    static __device__ __forceinline__ void run(const uint32_t (&raw)[32], int half, uint32_t (&code)[8], uint8_t &s)
+    {
+        const uint32_t am = wt_absmax2(raw);
+        const int sb = scale8_byte_from_f32_bits(half ? am & 0xFFFF0000u : am << 16);
+        const float inv = pow2_neg_e(sb);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            float y[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                y[i] = wt_value(raw[8 * g + i], half) * inv;
+            const uint2 c = e4m3x8(y);
+            code[2 * g] = c.x;
+            code[2 * g + 1] = c.y;
+        }
+        s = (uint8_t)sb;
+    }
+    static __device__ __forceinline__ int64_t scale_at(int64_t n, int64_t b, int64_t, int64_t kblocks)
+    {
+        return scale_index8<LAYOUT>(n, b, kblocks);
+    }
+    static __device__ __forceinline__ int64_t scale_count(int64_t pad_cols, int64_t kblocks) { return pad_cols * kblocks; }
+    static __device__ __forceinline__ bool in_bounds(int64_t, int64_t) { return true; }
+};
+
+// One thread per (column n, 32-block b) of W [K x N]: the form for odd N.
 template <int LAYOUT>
 __global__ void __launch_bounds__(256) weight_quant_mxfp8_kernel(const __nv_bfloat16 *__restrict__ w, int64_t K,
                                                                 int64_t N, int64_t Npad, uint8_t *__restrict__ codes,
@@ -593,6 +624,10 @@ cudaError_t launch_weight_quant_mxfp8(const void *w, int64_t K, int64_t N, void 
                                       cudaStream_t st)
 {
     const int64_t Npad = layout == RFQ_SCALE_MMA ? ((N + 127) / 128) * 128 : N;
+    if (N % 2 == 0)
+        return layout == RFQ_SCALE_MMA
+                   ? launch_weight_tile<WeightMxfp8<RFQ_SCALE_MMA>>(w, K, N, Npad, codes, scales, st)
+                   : launch_weight_tile<WeightMxfp8<RFQ_SCALE_ROWMAJOR>>(w, K, N, Npad, codes, scales, st);
     const int64_t work = Npad * (K / 32);
     const int blocks = (int)((work + 255) / 256);
     auto *wi = static_cast<const __nv_bfloat16 *>(w);
