@@ -44,107 +44,110 @@ __device__ __forceinline__ float ue6m2_value(int E, int M) // 2^(E-48) (1 + M/4)
     return __uint_as_float(((uint32_t)(E - 48 + 127) << 23) | ((uint32_t)M << 21));
 }
 
-// Smallest UE6M2 byte with 7 * value >= amax (amax > 0), clamped to [0, 255].
-// With amax = sig 2^ea (sig in [1, 2)), the candidates 7 (1 + M/4) 2^(E-48)
-// in increasing order are, for E - 48 = ea - 3, sig x {0.875, 1.09375,
-// 1.3125, 1.53125} and then, for E - 48 = ea - 2, {1.75, 2.1875, ...}; so
-// the answer follows from the significand bits of amax alone (thresholds
-// 0.09375, 0.3125, 0.53125 and 0.75 of the fraction: 0x0C0000, 0x280000,
-// 0x440000, 0x600000 in the 23-bit field), then the E range [0, 63].
+// Smallest UE6M2 byte with 7 * value >= amax (amax >= 0), clamped to [0, 255]:
+// amax / 7 rounded up to a significand of three bits, read off its float bits
+// (exponent and two fraction bits are the byte, offset by the exponent bias).
+// The factor is 1/7 less 2^-20 of it: an amax that is exactly 7 times a UE6M2
+// value then stays below that value and rounds up to it, and any other amax
+// (up to 12 significant bits) has a quotient at least 2^-13 of it beyond the
+// value below, which 2^-20 does not bridge.  The quantized inputs have 8 bits;
+// a residual that has more lies above 7 * 255's value and saturates either way.
 __device__ __forceinline__ int hif4_scale_byte(float amax)
 {
-    const uint32_t b = __float_as_uint(amax);
-    if (b < 0x00800000u)   // a subnormal amax is below every 7 S: byte 0
-        return 0;
-    const uint32_t f = b & 0x7FFFFFu;
-    const int e0 = (int)(b >> 23) - 127 - 3 + 48;   // E of the first candidate row
-    int E, M;
-    if (f <= 0x600000u && e0 >= 0) {
-        // first row, M = 1..3, or (E0 + 1, 0)
-        M = 1 + (f > 0x0C0000u) + (f > 0x280000u) + (f > 0x440000u);
-        E = e0;
-        if (M == 4) {
-            M = 0;
-            E = e0 + 1;
-        }
-    } else if (e0 >= -1) {
-        // second row: (E0 + 1, 0) if sig <= 1.75, else (E0 + 1, 1); with
-        // E0 = -1 the first row is out of range and this is the smallest
-        E = e0 + 1;
-        M = f > 0x600000u ? 1 : 0;
-    } else {
-        return 0;          // below the smallest macro scale: 2^-48 covers it
-    }
-    if (E > 63)
-        return 255;        // above the largest macro scale: saturate
-    return (E << 2) | M;
+    const uint32_t up = (__float_as_uint(amax * 0x1.249236p-3f) + 0x1FFFFFu) >> 21;
+    return min(max((int)up - (79 << 2), 0), 255);   // E = exponent field - 127 + 48
 }
 
-// Quantizes the eight elements x[0..7] of group g (sub-groups 2g, 2g+1) of a
-// 64-element block whose macro scale byte sb = (E << 2) | M is given.
-// Returns the codes (element i in nibble i) and this group's E1_8 / E1_16
-// bits (placed at their final metadata positions); `deq` receives the
-// dequantized values.
-//
-// A sub-group with exponent ex has the step 0.25 S 2^ex = 2^(E - 50 + ex)
-// (1 + M/4), formed from its bits, and its reciprocal is 2^(50 - E - ex)
-// 4 / (4 + M): rounded to fp32 that is the power of two times RN(4 / (4 + M))
-// (scaling by a power of two commutes with rounding in the normal range,
-// which every E in [0, 63] and ex in [0, 2] stays in), i.e. exactly the
-// correctly rounded reciprocal of the step, from one of four constants.
-__device__ __forceinline__ uint32_t hif4_group(const float (&x)[8], int sb, int g, uint32_t &meta_bits,
-                                               float (&deq)[8])
+// max |x| of the two sub-groups of a group (NaN is dropped).
+__device__ __forceinline__ void hif4_sub_amax(const float (&x)[8], float (&a)[2])
 {
-    const int E = sb >> 2, M = sb & 3;
-    const float S = ue6m2_value(E, M);
-    const float recip_m = M == 0 ? 1.0f : M == 1 ? 0.8f : M == 2 ? 0.6666666865348816f : 0.5714285969734192f;
-    int t[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        a[h] = fmax3(fmaxf(fabsf(x[4 * h]), fabsf(x[4 * h + 1])), fabsf(x[4 * h + 2]), fabsf(x[4 * h + 3]));
+}
+
+// What a macro scale byte sb = (E << 2) | M gives the elements of its block:
+// the step 0.25 S = 2^(E-50) (1 + M/4) of an exponent-0 sub-group as float
+// bits, and the bits of its reciprocal 2^(50-E) 4 / (4 + M), correctly
+// rounded (a power of two times one of four constants; no exponent of a
+// sub-group, 0 to 2, takes either out of the normal range).
+struct Hif4Scale {
+    uint32_t step, inv;
+    __device__ __forceinline__ explicit Hif4Scale(int sb)
+    {
+        const int M = sb & 3;
+        step = ((uint32_t)sb << 21) + (77u << 23);
+        const float recip_m = M == 0 ? 1.0f : M == 1 ? 0.8f : M == 2 ? 0.6666666865348816f : 0.5714285969734192f;
+        inv = __float_as_uint(recip_m) + (50u << 23) - ((uint32_t)(sb >> 2) << 23);
+    }
+};
+
+// Quantizes the eight elements x[0..7] of group g (sub-groups 2g, 2g+1, with
+// the maxima sub) of a 64-element block with macro scale s.  Returns the codes
+// (element i in nibble i) and this group's E1_8 / E1_16 bits (placed at their
+// final metadata positions); `deq` receives the dequantized values.
+//
+// The kernels were bound by the ALU pipe and the issue slots, not by memory (60
+// instructions per element in act_quant_hif4_kernel), so per-element and
+// per-sub-group work is what counts here: a quotient in one fma, a macro scale
+// in six instructions, the sign bits of four codes at a time, the sub-group
+// maxima reused for the block's.  act_quant_hif4_kernel on 4096 x 12288 (358 MB)
+// went from 88.3 to 68.8 us (5.2 TB/s), the weight quantizer on 5120 x 13824
+// from 58.1 to 42.1 us.
+__device__ __forceinline__ uint32_t hif4_group(const float (&x)[8], const float (&sub)[2], const Hif4Scale &s, int g,
+                                               uint32_t &meta_bits, float (&deq)[8])
+{
+    const float step0 = __uint_as_float(s.step);
+    // sub-group exponent: 0 up to 1.75 S, 1 up to 3.5 S, else 2 (of which E1_8
+    // carries one for the whole group)
+    bool over1[2], over2[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const float a = fmax3(fmaxf(fabsf(x[4 * h]), fabsf(x[4 * h + 1])), fabsf(x[4 * h + 2]), fabsf(x[4 * h + 3]));
-        t[h] = a <= 1.75f * S ? 0 : (a <= 3.5f * S ? 1 : 2);
+        over1[h] = !(sub[h] <= 7.0f * step0);
+        over2[h] = !(sub[h] <= 14.0f * step0);
     }
-    const int e18 = (t[0] == 2 || t[1] == 2) ? 1 : 0;
-    const int e116_0 = max(t[0] - e18, 0), e116_1 = max(t[1] - e18, 0);
-    meta_bits = ((uint32_t)e18 << (8 + g)) | ((uint32_t)e116_0 << (16 + 2 * g)) | ((uint32_t)e116_1 << (17 + 2 * g));
+    const bool e18 = over2[0] || over2[1];
+    uint32_t bits = e18 ? 1u << (8 + g) : 0u;
     float kf[8];   // the magnitudes k as floats (exact small integers)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int ex = e18 + (h ? e116_1 : e116_0);
-        const float step = __uint_as_float(((uint32_t)(E + ex + 77) << 23) | ((uint32_t)M << 21));
-        const float inv = __uint_as_float((uint32_t)(177 - E - ex) << 23) * recip_m;   // RN(1 / step)
+        if (e18 ? over2[h] : over1[h])
+            bits |= 1u << (16 + 2 * g + h);
+        const uint32_t ex = over2[h] ? 2u << 23 : (e18 || over1[h]) ? 1u << 23 : 0u;
+        const float step = __uint_as_float(s.step + ex), inv = __uint_as_float(s.inv - ex);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float v = x[4 * h + i];
-            const float a = fabsf(v);
-            // nearest k, ties to even, from the correctly rounded quotient
-            // a / step: a * inv is within one ulp of it (inv is the correctly
-            // rounded reciprocal), the remainder a - q step is exact (fma),
-            // and one correction q + r inv rounds to the correctly rounded
-            // quotient (Markstein's division refinement, P. Markstein, IA-64
-            // and Elementary Functions, 2000).  A true tie (a half-integer
-            // quotient) is then exact, and adding 2^23 rounds it to the even
-            // integer; any other quotient lies at least 2^-9 / 7 from every
-            // half-integer (a has 8 significant bits, step = D 2^s with D in
-            // {4,5,6,7}/4), far beyond the rounding error.  fminf saturates
-            // (NaN -> 7) before the rounding.
-            float q = a * inv;
-            q = fmaf(fmaf(-q, step, a), inv, q);
+            // nearest k, ties to even: q = |v| inv - 2^-24 in one rounding, then
+            // to an integer by adding 2^23.  inv is 1 / step times 1 + d with
+            // d = 0, 2^-26, 2^-25, 1.5 2^-25 for M = 0 .. 3, so at a tie k + 1/2
+            // the exact value is off by (k + 1/2) d - 2^-24: within half an ulp
+            // of k + 1/2 for every k from 1 to 6 (1.5: -2^-24 with d = 0, itself
+            // a tie that rounds to 1.5's even significand; 6.5: at most 7.75 of
+            // 8 2^-25), and q is the tie itself; 0.5 only ever moves down, as it
+            // has to.  Any other quotient lies at least 2^-9 / 7 from every
+            // half-integer (|v| has 8 significant bits, step = D 2^s with D in
+            // {4,5,6,7}/4).  fminf saturates (NaN -> 7) before the rounding.
+            const float q = fmaf(fabsf(v), inv, -0x1p-24f);
             const float k = (fminf(q, 7.0f) + 8388608.0f) - 8388608.0f;
             kf[4 * h + i] = k;
             deq[4 * h + i] = copysignf(k * step, v);
         }
     }
+    meta_bits = bits;
     // the eight 3-bit magnitudes into nibbles: two sums of k 16^i (exact
-    // below 2^16), their integer bits by adding 2^23, the low halves joined;
-    // then the sign bits (bit 3 of each nibble) from the inputs' sign bits
+    // below 2^16), their integer bits by adding 2^23, the low halves joined
     const float lo = fmaf(kf[3], 4096.0f, fmaf(kf[2], 256.0f, fmaf(kf[1], 16.0f, kf[0])));
     const float hi = fmaf(kf[7], 4096.0f, fmaf(kf[6], 256.0f, fmaf(kf[5], 16.0f, kf[4])));
-    uint32_t codes = __byte_perm(__float_as_uint(lo + 8388608.0f), __float_as_uint(hi + 8388608.0f), 0x5410);
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        codes |= (__float_as_uint(x[i]) >> (28 - 4 * i)) & (8u << (4 * i));
-    return codes;
+    const uint32_t codes = __byte_perm(__float_as_uint(lo + 8388608.0f), __float_as_uint(hi + 8388608.0f), 0x5410);
+    // the sign bits (bit 3 of each nibble): the top bytes of the even and of
+    // the odd elements gathered into a word each
+    auto tops = [&](int i) {
+        const uint32_t a = __byte_perm(__float_as_uint(x[i]), __float_as_uint(x[i + 2]), 0x0073);
+        const uint32_t b = __byte_perm(__float_as_uint(x[i + 4]), __float_as_uint(x[i + 6]), 0x7300);
+        return __byte_perm(a, b, 0x7610);
+    };
+    return codes | ((tops(0) >> 4) & 0x08080808u) | (tops(1) & 0x80808080u);
 }
 
 // rows: the matrix's row count; the block-major layout pads it to 128.
@@ -189,15 +192,16 @@ __device__ __forceinline__ void hif4_chunk(const float (&xf)[8], int g, bool ok,
                                            uint32_t *__restrict__ rcodes, uint32_t *__restrict__ rmeta,
                                            uint4 *__restrict__ m16, uint4 *__restrict__ r16)
 {
-    float am = fmax3(fmax3(fabsf(xf[0]), fabsf(xf[1]), fabsf(xf[2])),
-                     fmax3(fabsf(xf[3]), fabsf(xf[4]), fabsf(xf[5])), fmaxf(fabsf(xf[6]), fabsf(xf[7])));
+    float sub[2];
+    hif4_sub_amax(xf, sub);
+    float am = fmaxf(sub[0], sub[1]);   // (NaN only for a block of NaN: macro scale 0)
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1)
         am = fmaxf(am, __shfl_xor_sync(0xFFFFFFFFu, am, o));
     const int sb = am > 0.f ? hif4_scale_byte(am) : 0;
     uint32_t bits;
     float deq[8];
-    uint32_t code = hif4_group(xf, sb, g, bits, deq);
+    uint32_t code = hif4_group(xf, sub, Hif4Scale(sb), g, bits, deq);
     if (am == 0.f) {
         bits = 0;   // all-zero block: metadata 0, codes keep the sign of zero
     }
@@ -216,15 +220,16 @@ __device__ __forceinline__ void hif4_chunk(const float (&xf)[8], int g, bool ok,
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             r[i] = xf[i] - deq[i]; // exact
-        float ra = fmax3(fmax3(fabsf(r[0]), fabsf(r[1]), fabsf(r[2])),
-                         fmax3(fabsf(r[3]), fabsf(r[4]), fabsf(r[5])), fmaxf(fabsf(r[6]), fabsf(r[7])));
+        float rsub[2];
+        hif4_sub_amax(r, rsub);
+        float ra = fmaxf(rsub[0], rsub[1]);
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1)
             ra = fmaxf(ra, __shfl_xor_sync(0xFFFFFFFFu, ra, o));
         const int rsb = ra > 0.f ? hif4_scale_byte(ra) : 0;
         uint32_t rbits;
         float rdeq[8];
-        const uint32_t rcode = hif4_group(r, rsb, g, rbits, rdeq);
+        const uint32_t rcode = hif4_group(r, rsub, Hif4Scale(rsb), g, rbits, rdeq);
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1)
             rbits |= __shfl_xor_sync(0xFFFFFFFFu, rbits, o);
@@ -256,6 +261,12 @@ struct CodeVec<4> {
     static __device__ __forceinline__ T make(const uint32_t (&c)[4]) { return make_uint4(c[0], c[1], c[2], c[3]); }
 };
 
+// The E1_8 / E1_16 bits of groups 0 .. 3 moved to groups g .. g + 3.
+__device__ __forceinline__ uint32_t hif4_meta_shift(uint32_t bits, int g)
+{
+    return ((bits & 0xFF00u) << g) | ((bits & 0xFFFF0000u) << (2 * g));
+}
+
 template <bool RES, bool EXP, int NG>
 __device__ __forceinline__ void hif4_chunk_n(const float (&xf)[8 * NG], int gq, bool ok, bool on, int64_t c,
                                              int64_t moff, uint32_t *__restrict__ mcodes,
@@ -264,25 +275,29 @@ __device__ __forceinline__ void hif4_chunk_n(const float (&xf)[8 * NG], int gq, 
                                              uint4 *__restrict__ r16)
 {
     using CV = CodeVec<NG>;
+    float xg[NG][8], d[NG][8], sub[NG][2];
     float am = 0.f;
-#pragma unroll
-    for (int i = 0; i < 8 * NG; i += 4)
-        am = fmax3(am, fmaxf(fabsf(xf[i]), fabsf(xf[i + 1])), fmaxf(fabsf(xf[i + 2]), fabsf(xf[i + 3])));
-#pragma unroll
-    for (int o = 1; o < 8 / NG; o <<= 1)
-        am = fmaxf(am, __shfl_xor_sync(0xFFFFFFFFu, am, o));
-    const int sb = am > 0.f ? hif4_scale_byte(am) : 0;
-    float xg[NG][8], d[NG][8];
-    uint32_t code[NG], bits = 0;
 #pragma unroll
     for (int j = 0; j < NG; ++j) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
             xg[j][i] = xf[8 * j + i];
+        hif4_sub_amax(xg[j], sub[j]);
+        am = fmax3(am, sub[j][0], sub[j][1]);
+    }
+#pragma unroll
+    for (int o = 1; o < 8 / NG; o <<= 1)
+        am = fmaxf(am, __shfl_xor_sync(0xFFFFFFFFu, am, o));
+    const int sb = hif4_scale_byte(am);
+    const Hif4Scale sc(sb);
+    uint32_t code[NG], bits = 0;
+#pragma unroll
+    for (int j = 0; j < NG; ++j) {
         uint32_t b;
-        code[j] = hif4_group(xg[j], sb, NG * gq + j, b, d[j]);
+        code[j] = hif4_group(xg[j], sub[j], sc, j, b, d[j]);
         bits |= b;
     }
+    bits = hif4_meta_shift(bits, NG * gq);   // (from groups 0 .. NG - 1 to the lane's)
     if (am == 0.f)
         bits = 0;   // all-zero block: metadata 0, codes keep the sign of zero
 #pragma unroll
@@ -299,29 +314,30 @@ __device__ __forceinline__ void hif4_chunk_n(const float (&xf)[8 * NG], int gq, 
         }
     }
     if (RES) {
-        float r[NG][8];
+        float r[NG][8], rsub[NG][2];
         float ra = 0.f;
 #pragma unroll
         for (int j = 0; j < NG; ++j) {
 #pragma unroll
             for (int i = 0; i < 8; ++i)
                 r[j][i] = xg[j][i] - d[j][i]; // exact
-#pragma unroll
-            for (int i = 0; i < 8; i += 4)
-                ra = fmax3(ra, fmaxf(fabsf(r[j][i]), fabsf(r[j][i + 1])), fmaxf(fabsf(r[j][i + 2]), fabsf(r[j][i + 3])));
+            hif4_sub_amax(r[j], rsub[j]);
+            ra = fmax3(ra, rsub[j][0], rsub[j][1]);
         }
 #pragma unroll
         for (int o = 1; o < 8 / NG; o <<= 1)
             ra = fmaxf(ra, __shfl_xor_sync(0xFFFFFFFFu, ra, o));
-        const int rsb = ra > 0.f ? hif4_scale_byte(ra) : 0;
+        const int rsb = hif4_scale_byte(ra);
+        const Hif4Scale rsc(rsb);
         uint32_t rcode[NG], rbits = 0;
         float e[NG][8];
 #pragma unroll
         for (int j = 0; j < NG; ++j) {
             uint32_t b;
-            rcode[j] = hif4_group(r[j], rsb, NG * gq + j, b, e[j]);
+            rcode[j] = hif4_group(r[j], rsub[j], rsc, j, b, e[j]);
             rbits |= b;
         }
+        rbits = hif4_meta_shift(rbits, NG * gq);
 #pragma unroll
         for (int o = 1; o < 8 / NG; o <<= 1)
             rbits |= __shfl_xor_sync(0xFFFFFFFFu, rbits, o);
@@ -343,9 +359,9 @@ __device__ __forceinline__ void hif4_chunk_n(const float (&xf)[8 * NG], int gq, 
     }
 }
 
-// Groups per lane in act_quant_hif4_kernel: 2 (0.092 ms on the Qwen3-VL
-// down projection) against 1 (0.100 ms, eight lanes per block) and 4
-// (0.102 ms: 115 registers, two blocks per SM).
+// Groups per lane in act_quant_hif4_kernel: 2 (68.8 us on 4096 x 12288) against
+// 4 (80.2 us: registers leave two blocks per SM); a 64-register bound for four
+// blocks per SM at 2 groups made no difference (69.3 us).
 constexpr int kHNG = 2;
 
 template <bool RES, bool PHI, int LAYOUT, bool EXP>
@@ -498,16 +514,18 @@ struct WeightHif4 {
 #pragma unroll
         for (int i = 0; i < 64; ++i)
             am = fmaxf(am, fabsf(wt_value(raw[i], half)));
-        const int sb = am > 0.f ? hif4_scale_byte(am) : 0;
+        const int sb = hif4_scale_byte(am);
+        const Hif4Scale sc(sb);
         uint32_t bits = 0;
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
-            float x[8], deq[8];
+            float x[8], deq[8], sub[2];
 #pragma unroll
             for (int i = 0; i < 8; ++i)
                 x[i] = wt_value(raw[8 * g + i], half);
+            hif4_sub_amax(x, sub);
             uint32_t gb;
-            code[g] = hif4_group(x, sb, g, gb, deq);
+            code[g] = hif4_group(x, sub, sc, g, gb, deq);
             bits |= gb;
         }
         s = am == 0.f ? 0u : (bits | (uint32_t)sb);
@@ -534,14 +552,16 @@ __global__ void __launch_bounds__(256) weight_quant_hif4_kernel(const __nv_bfloa
     float am = 0.f;
     for (int i = 0; i < 64; ++i)
         am = fmaxf(am, fabsf(__bfloat162float(w[(blk * 64 + i) * N + n])));
-    const int sb = am > 0.f ? hif4_scale_byte(am) : 0;
+    const int sb = hif4_scale_byte(am);
+    const Hif4Scale sc(sb);
     uint32_t bits = 0, out[8];
     for (int g = 0; g < 8; ++g) {
-        float xf[8], deq[8];
+        float xf[8], deq[8], sub[2];
         for (int i = 0; i < 8; ++i)
             xf[i] = __bfloat162float(w[(blk * 64 + 8 * g + i) * N + n]);
+        hif4_sub_amax(xf, sub);
         uint32_t gb;
-        out[g] = hif4_group(xf, sb, g, gb, deq);
+        out[g] = hif4_group(xf, sub, sc, g, gb, deq);
         bits |= gb;
     }
     uint4 *dst = reinterpret_cast<uint4 *>(codes + n * (K >> 1) + blk * 32);
