@@ -172,17 +172,27 @@ __global__ void __launch_bounds__(256) phi_amax_kernel(const __nv_bfloat16 *__re
 
 // AMAX fallback (Sec. 4.3) for phi tiles of 128 rows x 256 columns, fused
 // into the quantizer: one block per tile stages the tile's 64 KB in shared
-// memory with cp.async (warp w holds rows 16w .. 16w + 15, lane l the l-th
-// 16-byte chunk of each; three blocks per SM), reduces max |x| over it (NaN
-// dropped, as by phi_amax_kernel), writes phi, then quantizes the tile.  A
-// phi = 0 tile's residual is written as zero codes and zero scales without
+// memory with cp.async (warp w holds rows R w .. R w + R - 1, lane l the l-th
+// 16-byte chunk of each; up to three blocks per SM), reduces max |x| over it
+// (NaN dropped, as by phi_amax_kernel), writes phi, then quantizes the tile.
+// A phi = 0 tile's residual is written as zero codes and zero scales without
 // being computed.  X is read from DRAM once, against twice for
 // phi_amax_kernel followed by act_quant_mxfp4_kernel.  (Measured slower:
 // the tile held in registers, two blocks per SM; splitting a tile over a
 // cluster of 2 or 4 blocks that exchange their maxima through distributed
 // shared memory; a persistent 512-thread form streaming the tiles through a
 // cp.async ring.)
-constexpr int kAmaxRows = 16; // rows per warp (8 warps = 128 rows)
+//
+// WARPS: with a few tiles per SM the time is one block's chain -- load, block
+// maximum, then each warp's rows one after another -- and 16 warps halve its
+// longest part.  8 / 16 / 32 warps, us: 18 x 7168 6.2 / 4.3 / 3.9, 300 x 5120
+// 7.4 / 5.6 / 5.6, 1777 x 5120 12.0 / 11.2 / 12.5, 8190 x 5120 33.8 / 32.0 / 42.9
+// (f = 0.47).  With many tiles the blocks of an SM cover for each other:
+// 32760 x 5120 112 / 108 / 151 at f = 0.47, but 97 / 100 / 146 with next to no
+// residual (three blocks of 8 warps per SM against two of 16), so beyond
+// kAmaxWideTiles tiles per SM the form with 8 warps keeps the call (at 8 tiles
+// per SM and next to no residual both take 29.5).
+constexpr int kAmaxWideTiles = 16;
 
 __device__ __forceinline__ void cp_async16_zfill(uint32_t saddr, const void *g, uint32_t src_bytes)
 {
@@ -199,14 +209,14 @@ __device__ __forceinline__ uint4 lds128(uint32_t saddr)
     return v;
 }
 
-template <int LAYOUT>
-__global__ void __launch_bounds__(256, 3)
+template <int LAYOUT, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, WARPS == 8 ? 3 : 2)
     act_quant_mxfp4_amax_kernel(const uint4 *__restrict__ x, int64_t M, int64_t K, uint32_t *__restrict__ mcodes,
                                 uint8_t *__restrict__ mscales, uint32_t *__restrict__ rcodes,
                                 uint8_t *__restrict__ rscales, uint8_t *__restrict__ phi, float tau)
 {
     grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
-    constexpr int R = kAmaxRows;
+    constexpr int R = 128 / WARPS;   // rows per warp
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t kchunks = K >> 3;
     const int kblocks = (int)(K >> 5);
@@ -239,14 +249,14 @@ __global__ void __launch_bounds__(256, 3)
             asm("max.bf16x2 %0, %1, %2;" : "=r"(acc) : "r"(acc), "r"(q[j] & 0x7fff7fffu));
     }
     const float am = fmaxf(__uint_as_float(acc << 16), __uint_as_float(acc & 0xffff0000u));
-    __shared__ uint32_t red[8];
+    __shared__ uint32_t red[WARPS];
     const uint32_t wmax = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(am)); // am >= 0: integer order
     if (lane == 0)
         red[warp] = wmax;
     __syncthreads();
     uint32_t tmax = red[0];
 #pragma unroll
-    for (int i = 1; i < 8; ++i)
+    for (int i = 1; i < WARPS; ++i)
         tmax = max(tmax, red[i]);
     const bool on = __uint_as_float(tmax) > tau;
     if (threadIdx.x == 0)
@@ -471,12 +481,15 @@ cudaError_t launch_act_quant_mxfp4(const void *x, int64_t M, int64_t K, int mode
         auto *rc = static_cast<uint32_t *>(rcodes);
         auto *rs = static_cast<uint8_t *>(rscales);
         constexpr int smem = 128 * 256 * 2;   // the tile, staged in shared memory
-        auto k = layout == RFQ_SCALE_MMA ? act_quant_mxfp4_amax_kernel<RFQ_SCALE_MMA>
-                                         : act_quant_mxfp4_amax_kernel<RFQ_SCALE_ROWMAJOR>;
+        const bool wide = (int64_t)tiles <= (int64_t)kAmaxWideTiles * num_sms();
+        auto k = layout == RFQ_SCALE_MMA ? (wide ? act_quant_mxfp4_amax_kernel<RFQ_SCALE_MMA, 16>
+                                                 : act_quant_mxfp4_amax_kernel<RFQ_SCALE_MMA, 8>)
+                                         : (wide ? act_quant_mxfp4_amax_kernel<RFQ_SCALE_ROWMAJOR, 16>
+                                                 : act_quant_mxfp4_amax_kernel<RFQ_SCALE_ROWMAJOR, 8>);
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess)
             return e;
-        k<<<tiles, 256, smem, st>>>(xi, M, K, mc, ms, rc, rs, phi, tau);
+        k<<<tiles, wide ? 512 : 256, smem, st>>>(xi, M, K, mc, ms, rc, rs, phi, tau);
         return cudaGetLastError();
     }
     if (mode == RFQ_FALLBACK_AMAX) {
