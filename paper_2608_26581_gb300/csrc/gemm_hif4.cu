@@ -588,7 +588,8 @@ cudaError_t launch_gemm_hif4(const GemmHif4Args &a, cudaStream_t st)
 {
     if (a.a_bf16) {
         // as for the MXFP4 GEMM: 32 x 12288 x 4096 takes 22 us there against
-        // 111 us here; 4096 rows stay here
+        // 111 us here, 1800 x 4096 x 1024 25.1 against 42.4; 4096 x 12288 x 4096
+        // stays here
         GemmSmallArgs s = {};
         s.x = a.a_codes;
         s.r = a.r_codes;
@@ -596,6 +597,7 @@ cudaError_t launch_gemm_hif4(const GemmHif4Args &a, cudaStream_t st)
         s.y = a.y;
         s.out_bf16 = a.out_bf16;
         s.residual = a.r_codes != nullptr;
+        s.phi = s.residual && a.phi != nullptr;
         s.bf16 = 1;
         s.M = a.M;
         s.N = a.N;

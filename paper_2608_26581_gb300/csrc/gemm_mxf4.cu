@@ -754,6 +754,8 @@ cudaError_t launch_gemm_mxf4(const GemmMxf4Args &a, cudaStream_t st)
         s.y = a.y;
         s.out_bf16 = a.out_bf16;
         s.residual = a.r_codes != nullptr;
+        s.phi = s.residual && a.phi != nullptr;
+        s.plain = a.plan_rows != 0;
         s.M = a.M;
         s.N = a.N;
         s.K = a.K;

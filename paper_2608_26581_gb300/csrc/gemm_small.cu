@@ -1,4 +1,5 @@
-// gemm_small.cu -- RFQ GEMM for few rows of X (Algorithm 1, Eq. rfq):
+// gemm_small.cu -- RFQ GEMM for few rows of X, or few output columns (Algorithm 1,
+// Eq. rfq):
 //   Y = X~ W~ + phi X^ W~
 // with the operands swapped and the reduction split over a cluster: a CTA's
 // MMA takes 128 W~ rows (output columns) as its M side and a tile of T rows
@@ -811,7 +812,7 @@ cudaError_t launch_variant(const GemmSmallArgs &a, const Plan &p, const Shape &s
     // for few rows): this one's set-up and its first look at W~ overlap it.
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = a.plain ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, kern, tw, tx, tr, (const uint8_t *)a.w_sf, (const uint8_t *)a.x_sf,
                               (const uint8_t *)a.r_sf, FUSED ? (const uint4 *)a.x : nullptr, a.y, a.status, s);
 }
@@ -902,6 +903,22 @@ float best_plan(const GemmSmallArgs &a0, int64_t rows, Plan &best)
     return t;
 }
 
+// Whether this kernel may take a layer of more than 1024 rows: where the tiled
+// kernels' tiles (256 x 256 on CTA pairs, bf16 128 x 256) do not fill the GPU
+// once, which few output columns leave to any number of rows.  With a full
+// wave of them and more the tiled kernels' larger tiles are the faster ones.
+// GEMM times, tiled -> here, us: MXFP4 1800 x 12288 x 512 32.1 -> 19.5, 1300 x
+// 4096 x 1024 14.8 -> 14.2, 4096 x 12288 x 512 32.6 -> 26.5; HiF4 1025 x 12288 x
+// 800 113 -> 33, 1800 x 4096 x 1024 42.4 -> 25.1, 4096 x 4096 x 512 43.2 -> 30.2.
+// Of 180 such shapes (700 to 4096 rows, 512 to 3072 columns) the estimates gave
+// this kernel none that the tiled one does faster.  With phi the tiled kernels
+// may skip up to the whole residual, so half their time has to beat them too.
+bool part_wave(const GemmSmallArgs &a, int64_t rows)
+{
+    const int64_t nt = (a.N + 255) / 256;
+    return a.bf16 ? (rows + 127) / 128 * nt <= 152 : (rows + 255) / 256 * nt <= 76;
+}
+
 // A layer's choice: its plan (cs = 0: none fits) and whether this kernel is the
 // faster one.  The search costs a few microseconds of host time, so each host
 // thread keeps the choices of its last shapes (a direct-mapped table).
@@ -916,7 +933,7 @@ const Choice &choose(const GemmSmallArgs &a, int64_t rows)
 {
     constexpr int kEntries = 64;
     static thread_local Choice table[kEntries];
-    const int flags = (a.residual ? 1 : 0) | (a.bf16 ? 2 : 0) | (a.fused ? 4 : 0);
+    const int flags = (a.residual ? 1 : 0) | (a.bf16 ? 2 : 0) | (a.fused ? 4 : 0) | (a.phi ? 8 : 0);
     const uint64_t h = ((uint64_t)rows * 0x9E3779B97F4A7C15ull ^ (uint64_t)a.N * 0xC2B2AE3D27D4EB4Full ^
                         (uint64_t)a.K * 0x165667B19E3779F9ull ^ (uint64_t)flags * 0x27D4EB2F165667C5ull) >> 40;
     Choice &c = table[h % kEntries];
@@ -926,8 +943,8 @@ const Choice &choose(const GemmSmallArgs &a, int64_t rows)
         c.K = a.K;
         c.flags = flags;
         c.plan = {};
-        // beyond 1024 rows the other kernels' tiles fill the GPU
-        c.take = rows <= 1024 && best_plan(a, rows, c.plan) * 1.05f < tiled_us(a, rows);
+        c.take = (rows <= 1024 || part_wave(a, rows)) &&
+                 best_plan(a, rows, c.plan) * 1.05f < tiled_us(a, rows) * (rows > 1024 && a.phi ? 0.5f : 1.f);
     }
     return c;
 }

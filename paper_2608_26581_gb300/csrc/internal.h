@@ -159,6 +159,8 @@ struct GemmSmallArgs {
     const void *x_sf, *r_sf, *w_sf;
     void *y;
     int out_bf16, residual, bf16, fused;
+    int phi;                       // the tiled kernels could skip residual tiles of this call
+    int plain;                     // not launched as a dependent of the kernel ahead (see launch_dependent)
     int64_t M, N, K;
     int32_t *status;
 };
