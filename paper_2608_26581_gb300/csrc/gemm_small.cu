@@ -904,19 +904,20 @@ float best_plan(const GemmSmallArgs &a0, int64_t rows, Plan &best)
 }
 
 // Whether this kernel may take a layer of more than 1024 rows: where the tiled
-// kernels' tiles (256 x 256 on CTA pairs, bf16 128 x 256) do not fill the GPU
-// once, which few output columns leave to any number of rows.  With a full
-// wave of them and more the tiled kernels' larger tiles are the faster ones.
+// kernels' tiles (256 x 256 on 76 CTA pairs, bf16 128 x 256 on 152 CTAs) make at
+// most three waves, so that a first or last wave that is nearly empty weighs.
 // GEMM times, tiled -> here, us: MXFP4 1800 x 12288 x 512 32.1 -> 19.5, 1300 x
-// 4096 x 1024 14.8 -> 14.2, 4096 x 12288 x 512 32.6 -> 26.5; HiF4 1025 x 12288 x
-// 800 113 -> 33, 1800 x 4096 x 1024 42.4 -> 25.1, 4096 x 4096 x 512 43.2 -> 30.2.
-// Of 180 such shapes (700 to 4096 rows, 512 to 3072 columns) the estimates gave
-// this kernel none that the tiled one does faster.  With phi the tiled kernels
-// may skip up to the whole residual, so half their time has to beat them too.
-bool part_wave(const GemmSmallArgs &a, int64_t rows)
+// 4096 x 1024 14.8 -> 14.2, 1025 x 4096 x 4096 24.4 -> 18.6, 1025 x 12288 x 4096
+// 58.4 -> 38.7; HiF4 1025 x 12288 x 800 113 -> 33, 1800 x 4096 x 1024 42.4 -> 25.1,
+// 1300 x 12288 x 4096 223 -> 157.  Of 276 such shapes (700 to 8190 rows, 512 to 7168
+// columns) the estimates gave this kernel none that the tiled one does faster,
+// and beyond two waves hardly any MXFP4 shape; with more waves the tiled kernels'
+// larger tiles are the faster ones.  With phi the tiled kernels may skip up to
+// the whole residual, so half their time has to be beaten.
+bool few_waves(const GemmSmallArgs &a, int64_t rows)
 {
     const int64_t nt = (a.N + 255) / 256;
-    return a.bf16 ? (rows + 127) / 128 * nt <= 152 : (rows + 255) / 256 * nt <= 76;
+    return a.bf16 ? (rows + 127) / 128 * nt <= 3 * 152 : (rows + 255) / 256 * nt <= 3 * 76;
 }
 
 // A layer's choice: its plan (cs = 0: none fits) and whether this kernel is the
@@ -943,7 +944,7 @@ const Choice &choose(const GemmSmallArgs &a, int64_t rows)
         c.K = a.K;
         c.flags = flags;
         c.plan = {};
-        c.take = (rows <= 1024 || part_wave(a, rows)) &&
+        c.take = (rows <= 1024 || few_waves(a, rows)) &&
                  best_plan(a, rows, c.plan) * 1.05f < tiled_us(a, rows) * (rows > 1024 && a.phi ? 0.5f : 1.f);
     }
     return c;

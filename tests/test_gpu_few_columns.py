@@ -53,3 +53,26 @@ def test_hif4(orc, M, K, N):
     assert rfq.rfq_workspace_status(ws) == rfq.RFQ_OK and bool((y[M] == 7.0).all())
     check_y(y[:M].double().cpu().numpy(),
             orc.linear(orc.FMT_HIF4, *qtensor_host(xq), *qtensor_host(xr), *qtensor_host(wq), M, K, N), bf16=True)
+
+
+# between one and three waves of the tiled kernels' tiles (taken: 80 and 96 tiles for 76 pairs, 180 for 152 CTAs)
+# and beyond three, against an fp64 product of the same operand values
+@pytest.mark.parametrize("fmt,M,K,N", [(F4, 1025, 4096, 4096), (F4, 1800, 1024, 2560), (F4, 5000, 384, 3600),
+                                       (H, 1025, 4096, 5120), (H, 2600, 4096, 2048), (H, 5000, 320, 3088)])
+def test_waves(fmt, M, K, N):
+    x, w = _inputs(M, K, N)
+    lay = MMA if fmt == F4 else rfq.RFQ_SCALE_ROWMAJOR
+    q = [rfq.empty_qtensor(fmt, lay, r, K) for r in (N, M, M)]
+    op = [rfq.empty_bf16_operand(r, K) for r in (N, M, M)]   # the exact values
+    rfq.rfq_quantize_weight(w, q[0])
+    rfq.rfq_quantize_act(x, q[1], q[2])
+    val = []
+    for t, o in zip(q, op):
+        rfq.rfq_dequant(t, o.codes)
+        val.append(o.codes.view(torch.bfloat16).view(t.rows, K).double())
+    y = torch.full((M + 1, N), float("nan"), device=DEV)
+    ws = torch.zeros(rfq.rfq_linear_workspace_bytes() // 4, dtype=torch.int32, device=DEV)
+    a = q if fmt == F4 else op
+    rfq.rfq_linear(a[1], a[2], None, 256, a[0], y[:M], rfq.RFQ_OUT_F32, ws)
+    assert rfq.rfq_workspace_status(ws) == rfq.RFQ_OK and bool(torch.isnan(y[M]).all())
+    check_y(y[:M].double().cpu().numpy(), ((val[1] + val[2]) @ val[0].t()).cpu().numpy())
