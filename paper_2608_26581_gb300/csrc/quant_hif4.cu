@@ -87,8 +87,8 @@ struct Hif4Scale {
 // (element i in nibble i) and this group's E1_8 / E1_16 bits (placed at their
 // final metadata positions); `deq` receives the dequantized values.
 //
-// The kernels were bound by the ALU pipe and the issue slots, not by memory (60
-// instructions per element in act_quant_hif4_kernel), so per-element and
+// The kernels were bound by the ALU pipe and the issue slots, not by memory (52
+// instructions per element in act_quant_hif4_kernel, 39 now), so per-element and
 // per-sub-group work is what counts here: a quotient in one fma, a macro scale
 // in six instructions, the sign bits of four codes at a time, the sub-group
 // maxima reused for the block's.  act_quant_hif4_kernel on 4096 x 12288 (358 MB)
