@@ -42,8 +42,9 @@
 //
 // Every mbarrier wait is bounded (kWaitLimitNs, or the limit in the caller's
 // workspace) and also gives up as soon as any CTA has recorded a timeout in
-// the caller's status word.  A CTA that gave up still meets its cluster at
-// both barriers, and no CTA of its cluster stores anything.
+// the caller's status word.  A CTA that gave up waits (bounded) for its copies
+// and MMAs in flight, whichever of its roles gave up and when, still meets its
+// cluster at both barriers, and no CTA of its cluster stores anything.
 #include <cuda_bf16.h>
 #include <cmath>
 #include <cstdint>
@@ -92,6 +93,7 @@ struct Ctl {
     uint32_t tmem_base;
     int32_t abort_flag;
     int32_t hold;                        // the workspace asks for a held start
+    int32_t issued, sf_issued;           // stages whose copies each producer issued (valid once its role ends)
 };
 constexpr size_t kCtlBytes = (sizeof(Ctl) + 1023) / 1024 * 1024;
 
@@ -138,13 +140,6 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t caddr)
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                  : "r"(caddr)
                  : "memory");
-    return v;
-}
-
-__device__ __forceinline__ int ld_cluster_s32(uint32_t caddr)
-{
-    int v;
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(caddr) : "memory");
     return v;
 }
 
@@ -197,6 +192,7 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
         }
         mbar_init(&S.acc_full, 1);
         mbar_init(&S.drain, 1);
+        S.issued = S.sf_issued = 0;
         fence_mbar_init();
     }
     if (threadIdx.x == 32 * SFP_WARP) {
@@ -278,10 +274,8 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
                     }
                 }
             }
-            if (stop || S.abort_flag)
-                // wait (bounded) until the copies in flight have landed
-                for (int q = max(0, p - ST); q < p; ++q)
-                    (void)wait_for(&S.full[q % ST], (q / ST) & 1, wl);
+            if (lane == 0)
+                S.issued = p;
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
@@ -357,15 +351,8 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
                     tc_commit(&S.empty[slot]);
                 }
             }
-            if (elect_one()) {
-                if (!stop)
-                    tc_commit(&S.acc_full);
-                if (S.abort_flag) {
-                    // wait (bounded) until every MMA issued above has completed
-                    tc_commit(&S.drain);
-                    (void)wait_for(&S.drain, 0, wl);
-                }
-            }
+            if (!stop && elect_one())
+                tc_commit(&S.acc_full);
         }
     } else if (warp < SFP_WARP) {
         // ------------------------------------------------ scale writers, then the epilogue
@@ -470,13 +457,14 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
                 // narrow tiles: the MMA thread's own work per stage is the bottleneck, so
                 // the operand tiles' barrier is waited for here; wide ones (SWAP, three
                 // stages in flight) wait for the two in parallel
-                if (!SWAP && !__all_sync(0xffffffffu, wait_for(&S.full[slot], par, wl, gstat))) {
+                const bool landed = SWAP || __all_sync(0xffffffffu, wait_for(&S.full[slot], par, wl, gstat));
+                tmem_st_wait();
+                if (!landed) {
                     if (lane == 0)
                         flag_timeout(S, status);
                     stop = true;
                     break;
                 }
-                tmem_st_wait();
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0)
@@ -575,9 +563,8 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
             }
             if (stop && lane == 0)
                 flag_timeout(S, status);
-            if (stop || S.abort_flag)
-                for (int q = max(0, p - ST); q < p; ++q)
-                    (void)wait_for(&S.sf_full[q % ST], (q / ST) & 1, wl);
+            if (lane == 0)
+                S.sf_issued = p;
         }
     } else if constexpr (FUSED) {
         // ------------------------------------------------ converters
@@ -649,6 +636,22 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
     // ---------------------------------------------------- cluster reduction
     tc_fence_before();
     __syncthreads();
+    if (S.abort_flag != 0 && !skip) {
+        // A role gave up, perhaps after the producers or the MMA issuer had
+        // ended theirs: what they have in flight still writes this CTA's shared
+        // and tensor memory, which its next owner gets when the CTA ends.
+        if (warp == 0 && lane == 0)
+            for (int q = max(0, S.issued - ST); q < S.issued; ++q)
+                (void)wait_for(&S.full[q % ST], (q / ST) & 1, wl);
+        if (warp == SFP_WARP && lane == 0)
+            for (int q = max(0, S.sf_issued - ST); q < S.sf_issued; ++q)
+                (void)wait_for(&S.sf_full[q % ST], (q / ST) & 1, wl);
+        if (warp == 1 && elect_one()) {  // (the lane that issued the MMAs: the election is the same each time)
+            tc_commit(&S.drain);
+            (void)wait_for(&S.drain, 0, wl);
+        }
+        __syncthreads();
+    }
     if (CS > 1)
         cluster_sync();                  // every CTA's partial tile is in its shared memory
     bool ok = true;

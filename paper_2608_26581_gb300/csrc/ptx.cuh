@@ -198,6 +198,14 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t saddr, uint32_t rank)
     return r;
 }
 
+// A word of a cluster CTA's shared memory, by its shared::cluster address.
+__device__ __forceinline__ int32_t ld_cluster_s32(uint32_t caddr)
+{
+    int32_t v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(caddr) : "memory");
+    return v;
+}
+
 // Relaxed arrive on the mbarrier at shared::cluster address `caddr`, in
 // another CTA of the cluster.  A release arrive at cluster scope stalls the
 // thread for hundreds of cycles; callers that need ordering complete their
