@@ -140,6 +140,8 @@ struct Smem {
     int32_t fq_last;              // fused quantizer: this CTA is the grid's last to finish
     uint64_t wait_ns;             // limit of the bounded waits (workspace word 1, else wl)
     int32_t abort_flag;
+    int32_t peer_abort;           // the other CTA of the pair gave up
+    int32_t issued, sf_issued;    // stages whose code / scale copies this CTA issued (valid once the role ends)
 };
 constexpr size_t kSmemBytes = sizeof(Smem) + 1024;
 static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
@@ -170,10 +172,45 @@ struct FqArgs {
     int ring;                     // slots of 256 rows in the scratch
 };
 
+// Tells the other CTA of the pair that this one gave up (a call: inlined, the
+// residual instantiations spill).
+__device__ __noinline__ void flag_peer(Smem &S)
+{
+    st_cluster_s32(mapa_shared(smem_u32(&S.peer_abort), cluster_ctarank() ^ 1), 1);
+}
+
 __device__ __forceinline__ void flag_timeout(Smem &S, int32_t *status)
 {
     S.abort_flag = 1;
+    flag_peer(S);
     atomicExch(status, kDevTimeout);
+}
+
+// Waits (bounded) for the copies that a pair of which a role gave up still has
+// in flight: they write shared memory that the next CTA gets when this one
+// ends.  The even CTA's barriers count the code copies of both CTAs; a stage
+// that only one of them issued never completes there, and one limit over all
+// stages outlasts its copies.  (A call, so that nothing of it takes registers
+// from the kernel's roles.)
+__device__ __noinline__ void settle_copies(Smem &S, bool mixed)
+{
+    const uint64_t limit = S.wait_ns;
+    if (threadIdx.x == 32 * SFP_WARP) {
+        for (int q = max(0, S.sf_issued - STAGES); q < S.sf_issued; ++q)
+            (void)mbar_wait(&S.sf_full[q % STAGES], (q / STAGES) & 1, limit);
+        if (mixed)
+            for (int q = max(0, S.issued - STAGES); q < S.issued; ++q)
+                (void)mbar_wait(&S.w4_full[q % STAGES], (q / STAGES) & 1, limit);
+    }
+    if (threadIdx.x == 0 && cluster_ctarank() == 0) {
+        const int n = max(S.issued, ld_cluster_s32(mapa_shared(smem_u32(&S.issued), 1)));
+        const uint64_t t0 = globaltimer_ns();
+        for (int q = max(0, n - STAGES); q < n; ++q) {
+            const uint64_t t = globaltimer_ns() - t0;
+            (void)mbar_wait(&S.full[q % STAGES], (q / STAGES) & 1, t < limit ? limit - t : 0);
+        }
+    }
+    __syncwarp();
 }
 
 // Where an output tile lives: the pair's first A row, the end of its rows
@@ -264,6 +301,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
             mbar_init(&S.phi_full[i], 32);
             mbar_init(&S.phi_empty[i], 2);   // (both producers)
         }
+        S.peer_abort = S.issued = S.sf_issued = 0;
         // A bounded wait of an earlier CTA or call gave up: skip the work
         // (both CTAs still meet at the cluster barriers).
         grid_dependency_wait();
@@ -336,6 +374,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
     const bool skip = S.abort_flag != 0 || (GRP && S.grp_bad != 0);
     const uint64_t wl = S.wait_ns;
     const int tiles = n_tiles * (GRP ? S.grp_pairs[G] : m_pairs);
+    if (threadIdx.x == 0 && S.abort_flag != 0)
+        flag_peer(S);                    // (its own look at the status word may have been earlier)
     auto coord = [&](int tile) {
         const int pi = tile / n_tiles, nt = tile - pi * n_tiles;
         TileCoord c;
@@ -512,19 +552,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
                     mbar_arrive(&S.phi_empty[r]);
                 }
             }
-            if (stop || S.abort_flag)
-                // wait (bounded) until the copies of the last stages landed: this
-                // CTA's scale atoms, or (even CTA) both CTAs' codes
-                for (int q = max(0, p - STAGES); q < p; ++q) {
-                    if (!OPS) {
-                        (void)mbar_wait(&S.sf_full[q % STAGES], (q / STAGES) & 1, wl);
-                        continue;
-                    }
-                    if (F8 == F8_MIXED)
-                        (void)mbar_wait(&S.w4_full[q % STAGES], (q / STAGES) & 1, wl);
-                    if (lead)
-                        (void)mbar_wait(&S.full[q % STAGES], (q / STAGES) & 1, wl);
-                }
+            (OPS ? S.issued : S.sf_issued) = p;
         }
     };
     if (warp == 0) {
@@ -983,6 +1011,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
                     // of the 128-byte swizzled row, from the 64-byte swizzled
                     // packed row (16-byte chunk j at j ^ ((row >> 1) & 3))
                     if (!__all_sync(0xffffffffu, mbar_wait(&S.w4_full[slot], (p / STAGES) & 1, wl, gstat))) {
+                        tmem_st_wait();
                         if (lane == 0)
                             flag_timeout(S, status);
                         stop = true;
@@ -1092,6 +1121,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
     tc_fence_before();
     __syncthreads();
     cluster_sync(); // the peer no longer signals this CTA, the pair's MMAs are complete
+    if (S.abort_flag != 0 || S.peer_abort != 0) {
+        // a role of either CTA gave up, perhaps after a producer had ended (both
+        // CTAs get here: each sets the other's peer_abort with its own flag)
+        settle_copies(S, F8 == F8_MIXED);
+        cluster_sync();
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc_pair(tmem, TMEM_COLS);

@@ -206,6 +206,11 @@ __device__ __forceinline__ int32_t ld_cluster_s32(uint32_t caddr)
     return v;
 }
 
+__device__ __forceinline__ void st_cluster_s32(uint32_t caddr, int32_t v)
+{
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(caddr), "r"(v) : "memory");
+}
+
 // Relaxed arrive on the mbarrier at shared::cluster address `caddr`, in
 // another CTA of the cluster.  A release arrive at cluster scope stalls the
 // thread for hundreds of cycles; callers that need ordering complete their

@@ -94,3 +94,39 @@ def test_cluster_split_fused(M):
     x, y = _x(M, K, M), torch.empty(M, N, device=DEV)
     _abort_then_compute(lambda ws: rfq.rfq_linear_fused(x, wq, y, rfq.RFQ_OUT_F32, ws), y,
                         lambda: rfq.fused_workspace(M, K))
+
+
+# ---- CTA pairs: both CTAs' copies complete on the even CTA's barriers
+
+@pytest.mark.parametrize("M,K,N", [(600, 640, 15360), (5000, 1024, 2048)])
+@pytest.mark.parametrize("tau", [None, 100.0])
+def test_pair(M, K, N, tau):
+    wq, xq, xr, y = _mxfp4(M, K, N)
+    phi = None
+    if tau is not None:
+        phi = torch.empty(-(-M // 128) * -(-K // 256), dtype=torch.uint8, device=DEV)
+        rfq.rfq_quantize_act(_x(M, K, M), xq, xr, phi, mode=rfq.RFQ_FALLBACK_AMAX, tau=tau)
+    _abort_then_compute(lambda ws: rfq.rfq_linear(xq, xr, phi, 256, wq, y, rfq.RFQ_OUT_F32, ws), y, _ws)
+
+
+def test_pair_mixed_rate():
+    M, K, N = 700, 512, 528
+    wq, xq, xr, y = _mxfp4(M, K, N, res_fmt=F8)
+    _abort_then_compute(lambda ws: rfq.rfq_linear_mixed(xq, xr, None, 256, wq, y, rfq.RFQ_OUT_F32, ws), y, _ws)
+
+
+def test_pair_e4m3():
+    M, K, N = 700, 512, 528
+    wq, x4, xr, y = _mxfp4(M, K, N, res_fmt=F8)
+    x8 = rfq.empty_qtensor(F8, MMA, M, K)
+    rfq.rfq_convert(x4, x8)
+    _abort_then_compute(lambda ws: rfq.rfq_linear(x8, xr, None, 256, wq, y, rfq.RFQ_OUT_F32, ws), y, _ws)
+
+
+def test_pair_fused():
+    M, K, N = 700, 1024, 1040
+    wq = rfq.empty_qtensor(F4, MMA, N, K)
+    rfq.rfq_quantize_weight(to_dev_bf16(make_weight(K, N, seed=N)), wq)
+    x, y = _x(M, K, M), torch.empty(M, N, device=DEV)
+    _abort_then_compute(lambda ws: rfq.rfq_linear_fused(x, wq, y, rfq.RFQ_OUT_F32, ws), y,
+                        lambda: rfq.fused_workspace(M, K))
