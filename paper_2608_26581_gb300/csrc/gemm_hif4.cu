@@ -337,10 +337,6 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
                 if (!stop)
                     tc_commit(&S.acc_full[buf]);
             }
-            if (S.abort_flag) {
-                tc_commit(&S.drain);
-                (void)mbar_wait(&S.drain, 0, wl);
-            }
         }
     } else if (warp < 2 + EPI_WARPS) {
         // ------------------------------------------------ epilogue (warps 2..5)
@@ -518,6 +514,12 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
         const int issued = S.issued;
         for (int p = max(0, issued - STAGES); p < issued; ++p)
             (void)mbar_wait(&S.full[p % STAGES], (p / STAGES) & 1, wl);
+    }
+    if (warp == 1 && S.abort_flag && elect_one()) {
+        // and until the MMAs issued above have completed: here, not at their issuer's
+        // end, since another role may have given up after it (the elected lane is the issuer)
+        tc_commit(&S.drain);
+        (void)mbar_wait(&S.drain, 0, wl);
     }
     __syncthreads();
     if (warp == 1) {

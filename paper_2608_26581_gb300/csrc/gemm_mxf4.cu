@@ -438,11 +438,6 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
                 if (!stop)
                     tc_commit(&S.acc_full);
             }
-            if (S.abort_flag) {
-                // wait (bounded) until every MMA issued above has completed
-                tc_commit(&S.drain);
-                (void)mbar_wait(&S.drain, 0, wl);
-            }
         }
     } else if (warp < 2 + EPI_WARPS) {
         // ------------------------------------------------ epilogue (warps 2..9)
@@ -700,6 +695,12 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
             (void)mbar_wait(&S.full[p % STAGES], (p / STAGES) & 1, wl);
             (void)mbar_wait(&S.sf_full[p % STAGES], (p / STAGES) & 1, wl);
         }
+    }
+    if (warp == 1 && S.abort_flag && elect_one()) {
+        // and until the MMAs issued above have completed: here, not at their issuer's
+        // end, since another role may have given up after it (the elected lane is the issuer)
+        tc_commit(&S.drain);
+        (void)mbar_wait(&S.drain, 0, wl);
     }
     __syncthreads();
     if (warp == 1) {

@@ -130,3 +130,25 @@ def test_pair_fused():
     x, y = _x(M, K, M), torch.empty(M, N, device=DEV)
     _abort_then_compute(lambda ws: rfq.rfq_linear_fused(x, wq, y, rfq.RFQ_OUT_F32, ws), y,
                         lambda: rfq.fused_workspace(M, K))
+
+
+# ---- single CTAs
+
+@pytest.mark.parametrize("counts", [[128, 384, 256], [2176, 2560]])   # (the second on CTA pairs)
+def test_grouped(counts):
+    K, N, M, G = 1024, 512, sum(counts), len(counts)
+    wq, xq, xr = rfq.empty_qtensor(F4, MMA, G * N, K), rfq.empty_qtensor(F4, MMA, M, K), rfq.empty_qtensor(F4, MMA, M, K)
+    rfq.rfq_quantize_weight(to_dev_bf16(np.concatenate([make_weight(K, N, seed=g) for g in range(G)], axis=1)), wq)
+    rfq.rfq_quantize_act(_x(M, K, M), xq, xr)
+    off = torch.from_numpy(np.cumsum([0] + counts).astype(np.int32)).to(DEV)
+    y = torch.empty(M, N, device=DEV)
+    _abort_then_compute(
+        lambda ws: rfq.rfq_linear_grouped(xq, xr, None, 256, off, wq, N, y, rfq.RFQ_OUT_F32, ws), y, _ws)
+
+
+@pytest.mark.parametrize("codes", [True, False])   # HiF4 expanded inside the GEMM; bf16 operands on whole tiles
+def test_hif4_tiled(codes):
+    M, K, N = 4096, 256, 4096
+    w16, xq, xr, xo, ro, y = _hif4(M, K, N)
+    a, r = (xq, xr) if codes else (xo, ro)
+    _abort_then_compute(lambda ws: rfq.rfq_linear(a, r, None, 256, w16, y, rfq.RFQ_OUT_F32, ws), y, _ws)
