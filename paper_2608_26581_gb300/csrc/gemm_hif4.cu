@@ -345,7 +345,8 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
         for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
             const int m_tile = tile / n_tiles, n_tile = tile - m_tile * n_tiles;
             const int buf = it & 1;
-            if (!mbar_wait(&S.acc_full[buf], (it >> 1) & 1, wl, gstat)) {
+            // warp-uniform outcome: the tcgen05 loads below need the whole warp
+            if (!__all_sync(0xffffffffu, mbar_wait(&S.acc_full[buf], (it >> 1) & 1, wl, gstat))) {
                 if (lane == 0)
                     flag_timeout(S, status);
                 break;
@@ -428,7 +429,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
                             dst[i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
                 }
             }
-            if (S.abort_flag)
+            if (__any_sync(0xffffffffu, S.abort_flag != 0))   // (the whole warp leaves or none of it)
                 break;
         }
         if (!CONV && lane == 0)
@@ -444,7 +445,8 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
         for (int tile = blockIdx.x; tile < tiles && !stop; tile += gridDim.x) {
             for (int ks = 0; ks < nks; ++ks, ++p) {
                 const int slot = p % STAGES;
-                if (!mbar_wait(&S.full[slot], (p / STAGES) & 1, wl, gstat)) {
+                // (warp-uniform outcome: the warp meets at the __syncwarp below)
+                if (!__all_sync(0xffffffffu, mbar_wait(&S.full[slot], (p / STAGES) & 1, wl, gstat))) {
                     if (lane == 0)
                         flag_timeout(S, status);
                     stop = true;

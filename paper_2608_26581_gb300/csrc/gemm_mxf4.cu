@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(PHI ? THREADS + 32 : THREADS, 1)
                     }
                 }
             }
-            if (S.abort_flag)
+            if (__any_sync(0xffffffffu, S.abort_flag != 0))   // (the whole warp leaves or none of it)
                 break;
         }
         if (lane == 0)

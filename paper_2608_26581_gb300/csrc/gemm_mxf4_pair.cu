@@ -935,7 +935,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
                     }
                 }
             }
-            if (S.abort_flag)
+            if (__any_sync(0xffffffffu, S.abort_flag != 0))   // (the whole warp leaves or none of it)
                 break;
         }
         if constexpr (FQ) {
