@@ -413,6 +413,44 @@ RFQ_API rfq_status rfq_linear_mixed(const rfq_qtensor *xq, const rfq_qtensor *xr
 RFQ_API rfq_status rfq_linear_profile(const rfq_qtensor *xq, const rfq_qtensor *xr, const rfq_qtensor *wq, void *y,
                                       int32_t out_dtype, void *workspace, void *stream);
 
+/* The GEMM kernels that rfq_linear chooses between. */
+typedef enum {
+    RFQ_KERNEL_AUTO = 0,   /* the one with the smaller estimated time */
+    RFQ_KERNEL_TILED = 1,  /* whole output tiles, one per CTA or CTA pair */
+    RFQ_KERNEL_CLUSTER = 2 /* small output tiles, the reduction split over a cluster's CTAs (MXFP4 operands,
+                              or bf16 expansions of HiF4) */
+} rfq_kernel;
+
+/* A layer's kernel and, for RFQ_KERNEL_CLUSTER, its launch shape. */
+typedef struct {
+    int32_t kernel;        /* RFQ_KERNEL_TILED or RFQ_KERNEL_CLUSTER */
+    int32_t cluster;       /* CTAs that share an output tile's reduction */
+    int32_t rows, cols;    /* rows of X and columns of Y per tile */
+    int32_t x_on_m;        /* 1: X is the MMA's 128-row operand; 0: W~ is */
+    int32_t joint;         /* 1: X~ and X^ side by side in one MMA */
+    int32_t ctas_per_sm;   /* 1 or 2 */
+    int32_t stages;        /* copy ring depth */
+    float cluster_us, tiled_us; /* the two estimates, in microseconds (0: not made) */
+} rfq_linear_plan;
+
+/* The kernel that rfq_linear takes for an M x K x N layer (host only, no
+ * device work; the choice depends on nothing else).  fmt: the activation's
+ * format, RFQ_FMT_MXFP4, RFQ_FMT_BF16 (expanded HiF4), RFQ_FMT_HIF4 or
+ * RFQ_FMT_MXFP8; residual: xr given; phi: phi given; fused: the layer goes
+ * through rfq_linear_fused instead.  kernel: RFQ_KERNEL_AUTO, or the kernel
+ * of an rfq_linear_on call.
+ * Errors: RFQ_ERR_INVALID_ARG, RFQ_ERR_SHAPE, RFQ_ERR_UNSUPPORTED (as
+ * rfq_linear_on). */
+RFQ_API rfq_status rfq_linear_choice(int32_t kernel, int64_t M, int64_t N, int64_t K, int32_t fmt, int32_t residual,
+                                     int32_t phi, int32_t fused, rfq_linear_plan *plan);
+
+/* rfq_linear on the given kernel whatever the estimate says: for tests and
+ * measurements.  RFQ_ERR_UNSUPPORTED: RFQ_KERNEL_CLUSTER for operands it does
+ * not take (MXFP8, unexpanded HiF4) or more than 65535 row tiles. */
+RFQ_API rfq_status rfq_linear_on(int32_t kernel, const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi,
+                                 int32_t phi_r_s, const rfq_qtensor *wq, void *y, int32_t out_dtype,
+                                 void *workspace, void *stream);
+
 /* The debug build (librfq_debug.so, compiled with -DRFQ_DEBUG_BOUNDS): the
  * activation and weight quantizers and the CTA-pair GEMM check the index of
  * every direct global store against its buffer's extent (codes, scales, the

@@ -440,9 +440,19 @@ rfq_status rfq_linear(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_
 } // extern "C"
 
 namespace rfq {
+namespace {
+// Operands that the cluster-split kernel can multiply (its grid's second
+// dimension counts 128-row tiles).
+bool cluster_kernel_takes(int32_t fmt, int64_t M)
+{
+    return (fmt == RFQ_FMT_MXFP4 || fmt == RFQ_FMT_BF16) && M <= (int64_t)65535 * 128;
+}
+bool kernel_ok(int32_t k) { return k == RFQ_KERNEL_AUTO || k == RFQ_KERNEL_TILED || k == RFQ_KERNEL_CLUSTER; }
+} // namespace
+
 rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
                        const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, void *stream,
-                       int64_t plan_rows)
+                       int64_t plan_rows, int kernel)
 {
     bool launch = false;
     const rfq_status s = linear_check(xq, xr, phi, phi_r_s, wq, y, out_dtype, workspace, &launch, true);
@@ -453,8 +463,11 @@ rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8
     const bool hif4 = xq->fmt == RFQ_FMT_HIF4 || bf16_act;
     const bool f8 = xq->fmt == RFQ_FMT_MXFP8;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (kernel == RFQ_KERNEL_CLUSTER && !cluster_kernel_takes(xq->fmt, M))
+        return RFQ_ERR_UNSUPPORTED;
     if (hif4) {
         GemmHif4Args a;
+        a.kernel = kernel;
         a.a_bf16 = bf16_act;
         a.a_codes = xq->codes;
         a.a_meta = xq->scales;
@@ -489,9 +502,53 @@ rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8
     a.f8 = f8;
     a.w4 = f8 && wq->fmt == RFQ_FMT_MXFP4;
     a.plan_rows = plan_rows;
+    a.kernel = kernel;
     return gemm_done(launch_gemm_mxf4(a, st), workspace, st);
 }
 } // namespace rfq
+
+extern "C" {
+
+rfq_status rfq_linear_on(int32_t kernel, const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi,
+                         int32_t phi_r_s, const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace,
+                         void *stream)
+{
+    if (!kernel_ok(kernel))
+        return RFQ_ERR_INVALID_ARG;
+    return linear_rows(xq, xr, phi, phi_r_s, wq, y, out_dtype, workspace, stream, 0, kernel);
+}
+
+rfq_status rfq_linear_choice(int32_t kernel, int64_t M, int64_t N, int64_t K, int32_t fmt, int32_t residual,
+                             int32_t phi, int32_t fused, rfq_linear_plan *plan)
+{
+    if (!plan || !kernel_ok(kernel) || !fmt_ok(fmt) || (fused && fmt != RFQ_FMT_MXFP4))
+        return RFQ_ERR_INVALID_ARG;
+    if (M < 1 || N < 1 || K < 1 || N % 16 != 0 || K % (fmt == RFQ_FMT_MXFP4 || fmt == RFQ_FMT_MXFP8 ? 128 : 64) != 0 ||
+        M > (int64_t)INT32_MAX || N > (int64_t)INT32_MAX || K > (int64_t)INT32_MAX)
+        return RFQ_ERR_SHAPE;
+    const bool can = cluster_kernel_takes(fmt, M) && (!fused || M <= 128);
+    if (kernel == RFQ_KERNEL_CLUSTER && !can)
+        return RFQ_ERR_UNSUPPORTED;
+    *plan = {};
+    plan->kernel = RFQ_KERNEL_TILED;
+    if (!can || kernel == RFQ_KERNEL_TILED)
+        return RFQ_OK;
+    GemmSmallArgs a = {};
+    a.residual = residual != 0;
+    a.phi = residual && phi;
+    a.bf16 = fmt == RFQ_FMT_BF16;
+    a.fused = fused != 0;
+    a.M = M;
+    a.N = N;
+    a.K = K;
+    if (fused || kernel == RFQ_KERNEL_CLUSTER || gemm_small_takes(a, M)) {
+        gemm_small_plan(a, M, *plan);
+        plan->kernel = RFQ_KERNEL_CLUSTER;
+    }
+    return RFQ_OK;
+}
+
+} // extern "C"
 
 namespace {
 // Workspace of rfq_linear_fused.  M <= 128 (the single-CTA fused kernel):

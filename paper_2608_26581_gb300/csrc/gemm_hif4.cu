@@ -607,7 +607,7 @@ cudaError_t launch_gemm_hif4(const GemmHif4Args &a, cudaStream_t st)
         s.N = a.N;
         s.K = a.K;
         s.status = a.status;
-        if (gemm_small_takes(s, a.M))
+        if (a.kernel == RFQ_KERNEL_CLUSTER || (a.kernel == RFQ_KERNEL_AUTO && gemm_small_takes(s, a.M)))
             return launch_gemm_small(s, a.M, st);
     }
     return a.a_bf16 ? launch_conv<false>(a, st) : launch_conv<true>(a, st);

@@ -762,7 +762,7 @@ cudaError_t launch_gemm_mxf4(const GemmMxf4Args &a, cudaStream_t st)
         s.K = a.K;
         s.status = a.status;
         const int64_t rows = a.plan_rows ? a.plan_rows : a.M;
-        if (gemm_small_takes(s, rows))
+        if (a.kernel == RFQ_KERNEL_CLUSTER || (a.kernel == RFQ_KERNEL_AUTO && gemm_small_takes(s, rows)))
             return launch_gemm_small(s, rows, st);
     }
     const bool grp_single = grp && !a.f8 && a.M < (int64_t)2048 * a.groups;

@@ -957,9 +957,38 @@ const Choice &choose(const GemmSmallArgs &a, int64_t rows)
 
 bool gemm_small_takes(const GemmSmallArgs &a, int64_t plan_rows) { return choose(a, plan_rows).take; }
 
+namespace {
+// (a layer that the choice never offers to this kernel has no plan in the table)
+Plan plan_of(const GemmSmallArgs &a, int64_t plan_rows)
+{
+    Plan p = choose(a, plan_rows).plan;
+    if (p.cs == 0)
+        best_plan(a, plan_rows, p);
+    return p;
+}
+} // namespace
+
+void gemm_small_plan(const GemmSmallArgs &a, int64_t plan_rows, rfq_linear_plan &out)
+{
+    const Plan p = plan_of(a, plan_rows);
+    Shape s;
+    out.cluster = 0;
+    out.tiled_us = a.fused ? 0.f : tiled_us(a, plan_rows);
+    if (p.cs == 0 || !make_shape(a, plan_rows, p, s))
+        return;
+    out.cluster = p.cs;
+    out.rows = s.T;
+    out.cols = s.NT;
+    out.x_on_m = p.nt > 0;
+    out.joint = s.cat;
+    out.ctas_per_sm = p.cols == 256 && !a.fused ? 2 : 1;
+    out.stages = s.stages;
+    out.cluster_us = plan_us(a, p, s);
+}
+
 cudaError_t launch_gemm_small(const GemmSmallArgs &a, int64_t plan_rows, cudaStream_t st)
 {
-    const Plan p = choose(a, plan_rows).plan;
+    const Plan p = plan_of(a, plan_rows);
     Shape s;
     if (p.cs == 0)
         return cudaErrorInvalidValue;

@@ -122,6 +122,7 @@ struct GemmMxf4Args {
     void *y;
     int out_bf16;
     int64_t M, N, K;
+    int kernel = RFQ_KERNEL_AUTO;              // the kernel to take (rfq_linear_on)
     int64_t plan_rows = 0;                     // rows of the whole matrix when M is a chunk of it in a call
                                                // from host memory (0: a device call on M rows)
     int32_t *status;
@@ -168,6 +169,7 @@ struct GemmSmallArgs {
 // rows of the whole matrix when a caller passes it in chunks: every chunk
 // then sums in the same order), and its launch.
 bool gemm_small_takes(const GemmSmallArgs &a, int64_t plan_rows);
+void gemm_small_plan(const GemmSmallArgs &a, int64_t plan_rows, rfq_linear_plan &out);   // (cluster 0: none fits)
 cudaError_t launch_gemm_small(const GemmSmallArgs &a, int64_t plan_rows, cudaStream_t st);
 
 // ---- HiF4 quantization (quant_hif4.cu); metadata layout RFQ_SCALE_MMA is
@@ -196,6 +198,7 @@ struct GemmHif4Args {
     int out_bf16;
     int64_t M, N, K;
     int32_t *status;
+    int kernel = RFQ_KERNEL_AUTO;    // the kernel to take (rfq_linear_on)
 };
 cudaError_t launch_gemm_hif4(const GemmHif4Args &a, cudaStream_t st);
 
@@ -227,7 +230,7 @@ rfq_status linear_check(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint
 // chunk's outputs are summed in the whole's order.
 rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8_t *phi, int32_t phi_r_s,
                        const rfq_qtensor *wq, void *y, int32_t out_dtype, void *workspace, void *stream,
-                       int64_t plan_rows);
+                       int64_t plan_rows, int kernel = RFQ_KERNEL_AUTO);
 
 // Blocks of `threads` threads (and `smem` dynamic shared bytes) of `kern`
 // resident on one SM at once (cached per kernel): grid-stride kernels launch

@@ -22,6 +22,7 @@ RFQ_FMT_MXFP4, RFQ_FMT_HIF4, RFQ_FMT_BF16, RFQ_FMT_MXFP8 = 0, 1, 2, 3
 RFQ_SCALE_ROWMAJOR, RFQ_SCALE_MMA = 0, 1
 RFQ_FALLBACK_NONE, RFQ_FALLBACK_ALL, RFQ_FALLBACK_AMAX = 0, 1, 2
 RFQ_OUT_F32, RFQ_OUT_BF16 = 0, 1
+RFQ_KERNEL_AUTO, RFQ_KERNEL_TILED, RFQ_KERNEL_CLUSTER = 0, 1, 2
 (RFQ_ERR_INVALID_ARG, RFQ_ERR_SHAPE, RFQ_ERR_ALIGNMENT, RFQ_ERR_UNSUPPORTED, RFQ_ERR_CUDA, RFQ_ERR_TIMEOUT,
  RFQ_ERR_DEVICE, RFQ_ERR_NONFINITE) = range(1, 9)
 STATUS_NAMES = {0: "RFQ_OK", 1: "RFQ_ERR_INVALID_ARG", 2: "RFQ_ERR_SHAPE", 3: "RFQ_ERR_ALIGNMENT",
@@ -32,7 +33,8 @@ EXPORTED = ("rfq_status_string", "rfq_qtensor_bytes", "rfq_quantize_weight", "rf
             "rfq_linear_workspace_bytes", "rfq_linear", "rfq_workspace_status", "rfq_dequant",
             "rfq_linear_noalloc", "rfq_linear_fused", "rfq_convert", "rfq_linear_grouped", "rfq_check_finite",
             "rfq_quantize_act_expand", "rfq_fp4_mma_peak", "rfq_linear_fused_workspace_bytes",
-            "rfq_linear_profile", "rfq_debug_bounds", "rfq_linear_mixed", "rfq_linear_host")
+            "rfq_linear_profile", "rfq_debug_bounds", "rfq_linear_mixed", "rfq_linear_host", "rfq_linear_on",
+            "rfq_linear_choice")
 
 
 class RFQError(RuntimeError):
@@ -77,6 +79,10 @@ def load_library(path: str = LIB_PATH):
         lib.rfq_linear_workspace_bytes.argtypes = []
         lib.rfq_linear.restype = I32
         lib.rfq_linear.argtypes = [QTP, QTP, P, I32, QTP, P, I32, P, P]
+        lib.rfq_linear_on.restype = I32
+        lib.rfq_linear_on.argtypes = [I32] + lib.rfq_linear.argtypes
+        lib.rfq_linear_choice.restype = I32
+        lib.rfq_linear_choice.argtypes = [I32, I64, I64, I64, I32, I32, I32, I32, P]
         lib.rfq_workspace_status.restype = I32
         lib.rfq_workspace_status.argtypes = [P, I32, P]
         lib.rfq_dequant.restype = I32
@@ -222,6 +228,26 @@ def rfq_linear(xq: QTensor, xr: QTensor | None, phi: torch.Tensor | None, phi_r_
     r = xr.packed() if xr is not None else None
     _check(load_library().rfq_linear(q, r, _ptr(phi), phi_r_s, w, _ptr(y), out_dtype, _ptr(workspace),
                                      _stream(stream)), "rfq_linear")
+
+
+def rfq_linear_on(kernel: int, xq: QTensor, xr: QTensor | None, phi: torch.Tensor | None, phi_r_s: int, wq: QTensor,
+                  y: torch.Tensor, out_dtype: int, workspace: torch.Tensor, stream=None):
+    """rfq_linear on the given kernel (RFQ_KERNEL_TILED, RFQ_KERNEL_CLUSTER): for tests and measurements."""
+    q, w = xq.packed(), wq.packed()
+    r = xr.packed() if xr is not None else None
+    _check(load_library().rfq_linear_on(kernel, q, r, _ptr(phi), phi_r_s, w, _ptr(y), out_dtype, _ptr(workspace),
+                                        _stream(stream)), "rfq_linear_on")
+
+
+_PLAN_KEYS = ("kernel", "cluster", "rows", "cols", "x_on_m", "joint", "ctas_per_sm", "stages", "cluster_us", "tiled_us")
+
+
+def rfq_linear_choice(M: int, N: int, K: int, fmt: int = RFQ_FMT_MXFP4, residual: bool = True, phi: bool = False,
+                      fused: bool = False, kernel: int = RFQ_KERNEL_AUTO) -> dict:
+    """The kernel and launch shape that rfq_linear takes for a layer (rfq_linear_plan in include/rfq.h); host only."""
+    buf = ctypes.create_string_buffer(struct.calcsize("@8i2f"))
+    _check(load_library().rfq_linear_choice(kernel, M, N, K, fmt, residual, phi, fused, buf), "rfq_linear_choice")
+    return dict(zip(_PLAN_KEYS, struct.unpack("@8i2f", buf)))
 
 
 def rfq_linear_mixed(xq: QTensor, xr: QTensor, phi: torch.Tensor | None, phi_r_s: int, wq: QTensor,

@@ -1,0 +1,46 @@
+"""rfq_linear_choice and rfq_linear_on on the host: what they refuse, and that every launch shape holds."""
+import random
+
+import pytest
+
+from paper_2608_26581_gb300 import _build, rfq
+
+F4, B16 = rfq.RFQ_FMT_MXFP4, rfq.RFQ_FMT_BF16
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    _build.build()
+    return rfq.load_library()
+
+
+def test_refusals():
+    for args, status in (((0, 16, 128), rfq.RFQ_ERR_SHAPE), ((1, 24, 128), rfq.RFQ_ERR_SHAPE),
+                         ((1, 16, 192), rfq.RFQ_ERR_SHAPE), ((1, 16, 96, B16), rfq.RFQ_ERR_SHAPE),
+                         ((1, 16, 128, 9), rfq.RFQ_ERR_INVALID_ARG),
+                         ((1, 16, 128, B16, True, False, True), rfq.RFQ_ERR_INVALID_ARG)):
+        with pytest.raises(rfq.RFQError) as e:
+            rfq.rfq_linear_choice(*args)
+        assert e.value.status == status
+    for fmt in (rfq.RFQ_FMT_MXFP8, rfq.RFQ_FMT_HIF4):
+        assert rfq.rfq_linear_choice(64, 256, 1024, fmt)["kernel"] == rfq.RFQ_KERNEL_TILED
+        with pytest.raises(rfq.RFQError) as e:
+            rfq.rfq_linear_choice(64, 256, 1024, fmt, kernel=rfq.RFQ_KERNEL_CLUSTER)
+        assert e.value.status == rfq.RFQ_ERR_UNSUPPORTED
+    assert rfq.load_library().rfq_linear_on(7, *[None] * 3, 256, *[None] * 2, 0, None, None) == rfq.RFQ_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("fmt", [F4, B16])
+def test_every_layer_has_a_launch_shape(fmt):
+    rng = random.Random(fmt)
+    for _ in range(3000):
+        M, N = max(1, int(2 ** rng.uniform(0, 15))), 16 * max(1, int(2 ** rng.uniform(0, 11)))
+        K = (128 if fmt == F4 else 64) * max(1, int(2 ** rng.uniform(0, 8)))
+        for res in (False, True):
+            p = rfq.rfq_linear_choice(M, N, K, fmt, res, kernel=rfq.RFQ_KERNEL_CLUSTER)
+            stages_k = -(-K // (256 if fmt == F4 else 64))
+            assert 1 <= p["cluster"] <= min(8, stages_k) and p["stages"] >= 2
+            assert p["rows"] % 16 == 0 and 16 <= p["rows"] <= 128 and p["cols"] % 16 == 0 and p["cols"] <= 256
+            # the chosen kernel is one of the two, and a cluster choice is the plan above
+            a = rfq.rfq_linear_choice(M, N, K, fmt, res)
+            assert a["kernel"] == rfq.RFQ_KERNEL_TILED or a == p
