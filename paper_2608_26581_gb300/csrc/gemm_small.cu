@@ -824,6 +824,25 @@ cudaError_t launch_variant(const GemmSmallArgs &a, const Plan &p, const Shape &s
 // columns) and two (256): cudaOccupancyMaxActiveClusters on a GB300.
 constexpr int kClusters[2][MAX_CLUSTER] = {{152, 76, 46, 36, 28, 23, 15, 15}, {304, 152, 97, 74, 58, 46, 38, 36}};
 
+// How a plan's tiles run: clusters in turn on the SMs, `share` CTAs of an SM at
+// once, n k-stages per CTA.
+struct Walk {
+    int tiles, waves, share, nks, n;
+};
+
+Walk walk_of(const GemmSmallArgs &a, const Plan &p, const Shape &s)
+{
+    Walk w;
+    w.tiles = (int)((a.N + s.NT - 1) / s.NT * ((a.M + s.T - 1) / s.T));
+    const bool two = p.cols == 256 && !a.fused;        // (the fused form's threads fill an SM)
+    const int cap = kClusters[two][p.cs - 1];
+    w.waves = (w.tiles + cap - 1) / cap;
+    w.share = two && w.tiles * p.cs > kClusters[0][0] ? 2 : 1;
+    w.nks = (int)((a.K + (a.bf16 ? 63 : 255)) / (a.bf16 ? 64 : 256));
+    w.n = (w.nks + p.cs - 1) / p.cs;
+    return w;
+}
+
 // Estimated microseconds of a plan.  The constants are a fit to the times of
 // 3,900 (shape, plan) pairs, M 8-900, K 1024-12288, N 1536-24576, both operand
 // kinds; choosing by it costs 2% on average against the best plan measured.
@@ -836,12 +855,8 @@ constexpr int kClusters[2][MAX_CLUSTER] = {{152, 76, 46, 36, 28, 23, 15, 15}, {3
 float plan_us(const GemmSmallArgs &a, const Plan &p, const Shape &s)
 {
     const bool f4 = !a.bf16, swap = p.nt > 0;
-    const int tiles = (int)((a.N + s.NT - 1) / s.NT * ((a.M + s.T - 1) / s.T));
-    const bool two = p.cols == 256 && !a.fused;        // (the fused form's threads fill an SM)
-    const int cap = kClusters[two][p.cs - 1];
-    const int waves = (tiles + cap - 1) / cap;
-    const int share = two && tiles * p.cs > kClusters[0][0] ? 2 : 1;
-    const int nks = (int)((a.K + (f4 ? 255 : 63)) / (f4 ? 256 : 64)), n = (nks + p.cs - 1) / p.cs;
+    const Walk w = walk_of(a, p, s);
+    const int waves = w.waves, share = w.share, n = w.n;
     const float xrows = a.fused ? 0.f : (float)(s.T * (s.res ? 2 : 1));
     const float kb = ((float)s.NT + xrows) / 8.f + (f4 ? (float)(s.w_atoms + (a.fused ? 0 : s.x_atoms * (s.res ? 2 : 1))) : 0.f);
     const int depth = s.stages * share;
@@ -872,6 +887,68 @@ float tiled_us(const GemmSmallArgs &a, int64_t rows)
     if (a.bf16)
         return 4.4f + waves * 0.58f * (a.K / 64);
     return 4.2f + waves * (0.63f + 0.35f * tiles / 152.f) * ((a.K + 255) / 256);
+}
+
+// The estimates above are for layers whose residual is multiplied in full; the
+// tiled kernels skip what is not there, and need a quarter less.  A layer
+// without a residual, or with phi (of which nothing is known here, so with no
+// tile kept, the tiled kernels' best), therefore has to pass a second
+// comparison, of estimates fitted to 2,144 layers of this kind timed on both
+// kernels, M 1-4096, K 512-13824, N 512-24576 (relative error 5%; bf16 7%):
+//   here   one + cluster cs + wave waves + kb (100 KB copied per SM, in turn) +
+//          hbm (MB of W~) + epi (10,000 outputs of a CTA, in turn) + moved (MB
+//          copied by all) + wide (stages of 256 W~ rows on the M side by 128
+//          rows of X, in turn)
+//   tiled  one + wave waves + k_wave (k-stages, in turn) + k_tile (k-stages
+//          times tiles per CTA or pair) + hbm
+// The margins are those with the fewest layers slower than on the other kernel.
+struct LightFit {
+    float one, cluster, wave, kb, hbm, epi, moved, wide;
+    struct Tiled {
+        float one, wave, k_wave, k_tile, hbm;
+    } pair, single;
+    float margin, slack;
+};
+constexpr LightFit kNoResidual[2] = {
+    {1.095f, 0.678f, 3.953f, 0.451f, 0.069f, 0.794f, 0.036f, 0.066f,
+     {5.215f, 1.042f, 0.276f, 0.054f, 0.086f}, {0.f, 4.151f, 0.391f, 0.f, 0.099f}, 0.97f, 0.3f},
+    {0.f, 0.468f, 5.747f, 0.396f, 0.087f, 0.469f, 0.027f, 0.121f,
+     {}, {4.657f, 0.078f, 0.346f, 0.065f, 0.066f}, 1.04f, 1.5f}};
+
+float light_plan_us(const GemmSmallArgs &a, const LightFit &f, const Plan &p, const Shape &s)
+{
+    const Walk w = walk_of(a, p, s);
+    const float kb = (float)(s.NT + s.T * (s.res ? 2 : 1)) / 8.f + (a.bf16 ? 0.f : 2.f);
+    const float in_turn = (float)(w.waves * w.n * w.share);
+    const bool wide = p.nt == 0 && s.NT == 2 * WROWS && !s.cat;
+    return f.one + (p.cs > 1 ? f.cluster * p.cs : 0.f) + f.wave * w.waves + f.kb * in_turn * kb / 100.f +
+           f.hbm * ((float)a.N * a.K * (a.bf16 ? 2.f : 0.53125f) / 1e6f) + f.epi * w.waves * s.T * s.NT / p.cs / 1e4f +
+           f.moved * ((float)w.tiles * w.nks * kb / 1e3f) + (wide ? f.wide * in_turn * s.T / 128.f : 0.f);
+}
+
+float light_tiled_us(const GemmSmallArgs &a, const LightFit &f, int64_t rows)
+{
+    const int64_t nt = (a.N + 255) / 256;
+    const bool pair = !a.bf16 && rows > 128;
+    const LightFit::Tiled &t = pair ? f.pair : f.single;
+    const int64_t tiles = pair ? (rows + 255) / 256 * nt : (rows + 127) / 128 * nt, at_once = pair ? 76 : 152;
+    const float waves = (float)((tiles + at_once - 1) / at_once), n = (float)((a.K + (a.bf16 ? 63 : 255)) / (a.bf16 ? 64 : 256));
+    return t.one + t.wave * waves + t.k_wave * waves * n + t.k_tile * n * tiles / at_once +
+           t.hbm * ((float)a.N * a.K * (a.bf16 ? 2.f : 0.53125f) / 1e6f);
+}
+
+// The second comparison, of a plan that the first one took.
+bool still_faster(const GemmSmallArgs &a0, int64_t rows, const Plan &p)
+{
+    if (a0.residual)
+        return true;
+    GemmSmallArgs a = a0;
+    a.M = rows;
+    Shape s;
+    if (!make_shape(a, rows, p, s))
+        return false;
+    const LightFit &f = kNoResidual[a.bf16 != 0];
+    return light_plan_us(a, f, p, s) * f.margin < light_tiled_us(a, f, rows) + f.slack;
 }
 
 // The fastest plan for a layer of `rows` rows; its estimate, or a huge number.
@@ -948,7 +1025,8 @@ const Choice &choose(const GemmSmallArgs &a, int64_t rows)
         c.flags = flags;
         c.plan = {};
         c.take = (rows <= 1024 || few_waves(a, rows)) &&
-                 best_plan(a, rows, c.plan) * 1.05f < tiled_us(a, rows) * (rows > 1024 && a.phi ? 0.5f : 1.f);
+                 best_plan(a, rows, c.plan) * 1.05f < tiled_us(a, rows) * (rows > 1024 && a.phi ? 0.5f : 1.f) &&
+                 still_faster(a, rows, c.plan);
     }
     return c;
 }

@@ -44,3 +44,24 @@ def test_every_layer_has_a_launch_shape(fmt):
             # the chosen kernel is one of the two, and a cluster choice is the plan above
             a = rfq.rfq_linear_choice(M, N, K, fmt, res)
             assert a["kernel"] == rfq.RFQ_KERNEL_TILED or a == p
+
+
+T, C = rfq.RFQ_KERNEL_TILED, rfq.RFQ_KERNEL_CLUSTER
+
+
+# layers timed on both kernels (quantizer + GEMM, us), apart by a tenth or more
+@pytest.mark.parametrize("fmt,M,K,N,kernel", [
+    (F4, 2500, 13824, 5120, T),    # 77 on the tiled kernel, 124 on the cluster-split one
+    (F4, 1777, 12288, 4096, T),    # 48, 74
+    (F4, 1000, 8192, 8192, T),     # 34, 46
+    (F4, 512, 5120, 13824, T),     # 24, 33
+    (F4, 16, 4096, 24576, T),      # 15.8, 19.9 (GEMM)
+    (F4, 128, 12288, 4096, C),     # 28, 14 (GEMM)
+    (F4, 256, 12288, 4096, C),     # 24, 19 (GEMM)
+    (B16, 64, 3584, 18944, T),     # 36, 51
+    (B16, 1777, 4096, 4096, T),    # 61, 83
+    (B16, 256, 13824, 5120, C),    # 93, 39 (GEMM)
+    (B16, 64, 8192, 8192, C),      # 59, 46 (GEMM)
+])
+def test_choice_without_a_residual(fmt, M, K, N, kernel):
+    assert rfq.rfq_linear_choice(M, N, K, fmt, residual=False)["kernel"] == kernel
