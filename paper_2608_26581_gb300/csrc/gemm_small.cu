@@ -914,6 +914,11 @@ constexpr LightFit kNoResidual[2] = {
      {5.215f, 1.042f, 0.276f, 0.054f, 0.086f}, {0.f, 4.151f, 0.391f, 0.f, 0.099f}, 0.97f, 0.3f},
     {0.f, 0.468f, 5.747f, 0.396f, 0.087f, 0.469f, 0.027f, 0.121f,
      {}, {4.657f, 0.078f, 0.346f, 0.065f, 0.066f}, 1.04f, 1.5f}};
+constexpr LightFit kPhi[2] = {
+    {1.283f, 0.63f, 3.62f, 0.321f, 0.081f, 0.954f, 0.042f, 0.043f,
+     {6.315f, 1.022f, 0.275f, 0.06f, 0.086f}, {0.f, 5.198f, 0.399f, 0.f, 0.096f}, 0.97f, 0.3f},
+    {0.f, 0.353f, 6.028f, 0.236f, 0.092f, 0.323f, 0.033f, 0.142f,
+     {}, {5.522f, 0.093f, 0.353f, 0.064f, 0.066f}, 1.02f, 1.f}};
 
 float light_plan_us(const GemmSmallArgs &a, const LightFit &f, const Plan &p, const Shape &s)
 {
@@ -940,14 +945,14 @@ float light_tiled_us(const GemmSmallArgs &a, const LightFit &f, int64_t rows)
 // The second comparison, of a plan that the first one took.
 bool still_faster(const GemmSmallArgs &a0, int64_t rows, const Plan &p)
 {
-    if (a0.residual)
+    if (a0.residual && !a0.phi)
         return true;
     GemmSmallArgs a = a0;
     a.M = rows;
     Shape s;
     if (!make_shape(a, rows, p, s))
         return false;
-    const LightFit &f = kNoResidual[a.bf16 != 0];
+    const LightFit &f = (a.phi ? kPhi : kNoResidual)[a.bf16 != 0];
     return light_plan_us(a, f, p, s) * f.margin < light_tiled_us(a, f, rows) + f.slack;
 }
 

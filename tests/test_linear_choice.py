@@ -65,3 +65,17 @@ T, C = rfq.RFQ_KERNEL_TILED, rfq.RFQ_KERNEL_CLUSTER
 ])
 def test_choice_without_a_residual(fmt, M, K, N, kernel):
     assert rfq.rfq_linear_choice(M, N, K, fmt, residual=False)["kernel"] == kernel
+
+
+# with phi 0 on every tile, where the tiled kernels do least
+@pytest.mark.parametrize("fmt,M,K,N,kernel", [
+    (F4, 1000, 13824, 5120, T),    # 55, 71
+    (F4, 400, 13824, 5120, T),     # 33, 38
+    (F4, 128, 12288, 4096, C),     # 37, 17
+    (F4, 256, 12288, 4096, C),     # 33, 23
+    (B16, 333, 5120, 13824, T),    # 82, 96
+    (B16, 300, 5120, 13824, T),    # 82, 95
+    (B16, 256, 12288, 4096, C),    # 96, 44
+])
+def test_choice_with_phi(fmt, M, K, N, kernel):
+    assert rfq.rfq_linear_choice(M, N, K, fmt, phi=True)["kernel"] == kernel
