@@ -919,6 +919,11 @@ constexpr LightFit kPhi[2] = {
      {6.315f, 1.022f, 0.275f, 0.06f, 0.086f}, {0.f, 5.198f, 0.399f, 0.f, 0.096f}, 0.97f, 0.3f},
     {0.f, 0.353f, 6.028f, 0.236f, 0.092f, 0.323f, 0.033f, 0.142f,
      {}, {5.522f, 0.093f, 0.353f, 0.064f, 0.066f}, 1.02f, 1.f}};
+// bf16 operands with the whole residual, up to 128 rows: the first comparison
+// underrates what a split reduction costs where W~ (2 bytes an element) comes
+// from HBM.  32 x 3584 x 18944: 48.5 us here against 43.5.
+constexpr LightFit kBf16Decode = {0.f, 0.353f, 6.028f, 0.236f, 0.092f, 0.323f, 0.033f, 0.142f,
+                                  {}, {5.39f, 0.244f, 0.513f, 0.067f, 0.037f}, 1.02f, 0.f};
 
 float light_plan_us(const GemmSmallArgs &a, const LightFit &f, const Plan &p, const Shape &s)
 {
@@ -945,14 +950,15 @@ float light_tiled_us(const GemmSmallArgs &a, const LightFit &f, int64_t rows)
 // The second comparison, of a plan that the first one took.
 bool still_faster(const GemmSmallArgs &a0, int64_t rows, const Plan &p)
 {
-    if (a0.residual && !a0.phi)
+    const bool full = a0.residual && !a0.phi;
+    if (full && (!a0.bf16 || rows > 128))
         return true;
     GemmSmallArgs a = a0;
     a.M = rows;
     Shape s;
     if (!make_shape(a, rows, p, s))
         return false;
-    const LightFit &f = (a.phi ? kPhi : kNoResidual)[a.bf16 != 0];
+    const LightFit &f = full ? kBf16Decode : (a.phi ? kPhi : kNoResidual)[a.bf16 != 0];
     return light_plan_us(a, f, p, s) * f.margin < light_tiled_us(a, f, rows) + f.slack;
 }
 

@@ -79,3 +79,9 @@ def test_choice_without_a_residual(fmt, M, K, N, kernel):
 ])
 def test_choice_with_phi(fmt, M, K, N, kernel):
     assert rfq.rfq_linear_choice(M, N, K, fmt, phi=True)["kernel"] == kernel
+
+
+@pytest.mark.parametrize("M,K,N,kernel", [(32, 3584, 18944, T),     # 43.5, 48.5
+                                          (32, 12288, 4096, C)])    # 111, 22 (GEMM)
+def test_choice_bf16_decode(M, K, N, kernel):
+    assert rfq.rfq_linear_choice(M, N, K, B16)["kernel"] == kernel
