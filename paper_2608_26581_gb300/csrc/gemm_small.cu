@@ -572,12 +572,20 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
         // (row lane / 8 of the step, block lane % 8); a stage has T / 4 steps,
         // dealt to the warps in order over all stages.  The next step's loads
         // are issued before this one waits for its stage's buffers.
-        const int steps = T / 4, total = n_st * steps;
+        // (a warp's place, stage and step in it, is counted on: with divisions by
+        // steps and the ring's length it was a third of a step without a residual)
+        const int steps = T / 4;
         const int kb = sh.K >> 5;
-        auto load = [&](int u, uint32_t (&w)[16]) {
-            const int p = u / steps;
-            const int m = (u - p * steps) * 4 + (lane >> 3), b = (k_lo + p) * 8 + (lane & 7);
-            if (u < total && m < sh.M && b < kb) {
+        struct Place {
+            int p, i;                    // k-stage, step
+        };
+        auto forth = [&](Place &at) {
+            for (at.i += CONV_WARPS; at.i >= steps; at.i -= steps)
+                ++at.p;
+        };
+        auto load = [&](const Place &at, uint32_t (&w)[16]) {
+            const int m = at.i * 4 + (lane >> 3), b = (k_lo + at.p) * 8 + (lane & 7);
+            if (at.p < n_st && m < sh.M && b < kb) {
                 const uint4 *px = xbf + (int64_t)m * (sh.K >> 3) + (int64_t)b * 4;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -594,19 +602,28 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
             }
         };
         uint32_t cur[16], nxt[16];
-        int u = warp - CONV_WARP0;
-        load(u, cur);
-        for (; u < total && !skip; u += CONV_WARPS) {
-            load(u + CONV_WARPS, nxt);
-            const int p = u / steps, slot = p % ST;
-            if (!__all_sync(0xffffffffu, wait_for(&S.empty[slot], ((p / ST) & 1) ^ 1, wl, gstat))) {
+        Place now = {0, warp - CONV_WARP0 - CONV_WARPS}, ahead;
+        forth(now);
+        load(now, cur);
+        int slot = 0, slot_p = 0;        // ring slot of stage slot_p, and its phase
+        uint32_t phase = 0;
+        for (; now.p < n_st && !skip; now = ahead) {
+            ahead = now;
+            forth(ahead);
+            load(ahead, nxt);
+            for (; slot_p < now.p; ++slot_p)
+                if (++slot == ST) {
+                    slot = 0;
+                    phase ^= 1;
+                }
+            if (!__all_sync(0xffffffffu, wait_for(&S.empty[slot], phase ^ 1, wl, gstat))) {
                 if (lane == 0)
                     flag_timeout(S, status);
                 break;
             }
             float xf[32];
             bf16x32_to_f32(cur, xf);
-            const int r = (u - p * steps) * 4 + (lane >> 3), b = lane & 7;
+            const int r = now.i * 4 + (lane >> 3), b = lane & 7;
             uint8_t *st = ring + slot * sh.stage_bytes;
             uint8_t *sx = st + sh.sf_off + sh.w_atoms * 2 * ATOM, *sr = sx + 2 * ATOM;
             const int co = r * ROW + ((b ^ (r & 7)) << 4);   // 128-byte swizzle
@@ -867,7 +884,9 @@ float plan_us(const GemmSmallArgs &a, const Plan &p, const Shape &s)
                              : 4.f * (s.res ? 2 : 1) * p.wt * mma((float)s.T);
     per = fmaxf(per, c * share / 1900.f);
     if (a.fused)
-        per = fmaxf(per, 0.93f * s.T / (4.f * CONV_WARPS));   // a converter warp's step: four rows
+        // a converter warp's step (four rows): 0.93 us while its stage's other waits show,
+        // beyond 64 rows, where its steps follow one another, 0.78, without a residual 0.57
+        per = fmaxf(per, (s.T <= 64 ? 0.93f : s.res ? 0.78f : 0.57f) * s.T / (4.f * CONV_WARPS));
     const float t = 0.6f + (p.cs > 1 ? 0.4f * p.cs : 0.f) +
                     waves * (4.8f + n * per + 0.73e-4f * s.T * s.NT / p.cs);
     const float hbm = (float)a.N * a.K * (f4 ? 0.53125f : 2.f) / 5.1e6f;

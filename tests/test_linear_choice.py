@@ -85,3 +85,9 @@ def test_choice_with_phi(fmt, M, K, N, kernel):
                                           (32, 12288, 4096, C)])    # 111, 22 (GEMM)
 def test_choice_bf16_decode(M, K, N, kernel):
     assert rfq.rfq_linear_choice(M, N, K, B16)["kernel"] == kernel
+
+
+# 128 rows quantized inside the GEMM: 96 tiles in one wave of single CTAs take 40.6 us, in three waves of clusters of
+# four 59.8
+def test_fused_wide_layer_is_one_wave():
+    assert rfq.rfq_linear_choice(128, 24576, 4096, residual=False, fused=True)["cluster"] == 1
