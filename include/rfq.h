@@ -452,9 +452,9 @@ RFQ_API rfq_status rfq_linear_on(int32_t kernel, const rfq_qtensor *xq, const rf
                                  void *workspace, void *stream);
 
 /* The debug build (librfq_debug.so, compiled with -DRFQ_DEBUG_BOUNDS): the
- * activation and weight quantizers and the CTA-pair GEMM check the index of
- * every direct global store against its buffer's extent (codes, scales, the
- * fused quantizer's ring, the grouped GEMM's row stores); an out-of-range
+ * MXFP4 quantizers, the CTA-pair GEMM and the cluster-split GEMM check the
+ * index of every direct global store against its buffer's extent (codes,
+ * scales, the fused quantizer's ring, rows of Y); an out-of-range
  * store is skipped and the source line of the first one is recorded.  This
  * call synchronizes the device and reports it: RFQ_OK (none, *line = 0) or
  * RFQ_ERR_SHAPE with *line set; clear != 0 resets the records.  The normal

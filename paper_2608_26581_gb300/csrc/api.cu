@@ -771,7 +771,8 @@ rfq_status rfq_debug_bounds(int32_t *line, int32_t clear)
         return RFQ_ERR_INVALID_ARG;
     if (cudaDeviceSynchronize() != cudaSuccess)
         return RFQ_ERR_CUDA;
-    const int words[2] = {debug_word_quant_mxfp4(clear), debug_word_gemm_mxf4_pair(clear)};
+    const int words[3] = {debug_word_quant_mxfp4(clear), debug_word_gemm_mxf4_pair(clear),
+                          debug_word_gemm_small(clear)};
     *line = 0;
     for (int w : words) {
         if (w < 0)

@@ -55,6 +55,7 @@
 
 namespace rfq {
 namespace {
+RFQ_DEBUG_WORD_DECL
 
 constexpr int WROWS = 128;               // W~ rows per MMA
 constexpr int ROW = 128;                 // operand bytes per row per stage
@@ -572,8 +573,8 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
         // (row lane / 8 of the step, block lane % 8); a stage has T / 4 steps,
         // dealt to the warps in order over all stages.  The next step's loads
         // are issued before this one waits for its stage's buffers.
-        // (a warp's place, stage and step in it, is counted on: with divisions by
-        // steps and the ring's length it was a third of a step without a residual)
+        // A warp's place, stage and step in it, is counted on (128 x 4096 x 24576
+        // without a residual: 56.0 us; dividing by steps and the ring's length 59.8).
         const int steps = T / 4;
         const int kb = sh.K >> 5;
         struct Place {
@@ -715,6 +716,8 @@ __global__ void __launch_bounds__(FUSED ? 32 * (CONV_WARP0 + CONV_WARPS) : 32 * 
                             a.w += v[j][u].w;
                         }
                     const int64_t at = (int64_t)(t0 + t) * sh.N + n;
+                    if (!RFQ_IN_BOUNDS(at + 3, (int64_t)sh.M * sh.N))
+                        continue;
                     if (sh.out_bf16) {
                         const __nv_bfloat162 b0 = __floats2bfloat162_rn(a.x, a.y), b1 = __floats2bfloat162_rn(a.z, a.w);
                         *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(y) + at) = make_uint2(
@@ -1111,5 +1114,7 @@ cudaError_t launch_gemm_small(const GemmSmallArgs &a, int64_t plan_rows, cudaStr
         return p.wt == 2 ? launch_variant<true, true, 2>(a, p, s, st) : launch_variant<true, true, 1>(a, p, s, st);
     return p.wt == 2 ? launch_variant<true, false, 2>(a, p, s, st) : launch_variant<true, false, 1>(a, p, s, st);
 }
+
+RFQ_DEBUG_WORD_ACCESSOR(debug_word_gemm_small)
 
 } // namespace rfq

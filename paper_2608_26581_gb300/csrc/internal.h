@@ -48,6 +48,7 @@ __device__ __forceinline__ bool debug_in_bounds(int64_t i, int64_t n, int line, 
 // of the first out-of-range store, 0 if none; -1 if it cannot be read).
 int debug_word_quant_mxfp4(int clear);
 int debug_word_gemm_mxf4_pair(int clear);
+int debug_word_gemm_small(int clear);
 
 // Device status word values written into a workspace by kernels.
 constexpr int32_t kDevOk = 0;

@@ -55,3 +55,14 @@ def test_form(fmt, M, K, N, res, form):
     rfq.rfq_linear_on(rfq.RFQ_KERNEL_CLUSTER, a[1], a[2] if res else None, None, 256, a[0], y[:M], rfq.RFQ_OUT_F32, ws)
     assert rfq.rfq_workspace_status(ws) == rfq.RFQ_OK and bool(torch.isnan(y[M]).all())
     check_y(y[:M].double().cpu().numpy(), ((xv + rv if res else xv) @ w.t()).cpu().numpy())
+
+
+def test_debug_build_checks_the_stores(tmp_path, monkeypatch):
+    """The debug build's bounds checks on this kernel's ragged stores."""
+    import test_gpu_debug_build as dbg
+    cases = dbg._CASES.replace("rfq.rfq_linear(xq", "rfq.rfq_linear_on(rfq.RFQ_KERNEL_CLUSTER, xq")
+    fused = "\nyf = torch.zeros(100, N, device='cuda')\n" \
+            "rfq.rfq_linear_fused(x[:100].contiguous(), wq, yf, rfq.RFQ_OUT_F32, rfq.fused_workspace(100, K)); keep(yf)\n"
+    assert "RFQ_KERNEL_CLUSTER" in cases and "# grouped" in cases
+    monkeypatch.setattr(dbg, "_CASES", cases.replace("# grouped", fused + "# grouped"))
+    dbg.test_debug_build_records_no_out_of_range_store_and_matches(tmp_path)
