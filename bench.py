@@ -759,13 +759,15 @@ def run_rfq(args):
         t_peak, t_peak_sust = pk["bf16_burst"] * FP4_OVER_BF16, pk["bf16_sust"] * FP4_OVER_BF16
         t_src = (f"{pk['src']} bf16 burst {pk['bf16_burst']} TFLOP/s x {FP4_OVER_BF16:g} "
                  f"(nominal dense FP4/BF16 ratio), of {pk['src']}")
-        # CTA pairs beyond one 128-row tile (the workloads of few rows may take
-        # gemm_small_kernel instead: the library chooses by estimated time); grouped launches whose groups
+        # CTA pairs beyond one 128-row tile; grouped launches whose groups
         # average under 2048 stacked rows run 128-row tiles on single CTAs
-        grouped_single = grouped and Mb < 2048 * spec.groups
         # (fused: CTA pairs with the quantizer in their epilogue warps beyond 128 rows)
-        t_kernel = ("gemm_mxf4_pair_kernel" if M > 128 else "gemm_small_kernel") if fused else (
-            "gemm_mxf4_kernel" if M <= 128 or grouped_single else "gemm_mxf4_pair_kernel")
+        t_kernel = "gemm_mxf4_kernel" if M <= 128 or grouped and Mb < 2048 * spec.groups else "gemm_mxf4_pair_kernel"
+    # (the library's own choice, by estimated time, for the rows of one call)
+    if not (quant_only or f8 or grouped) and rfq.rfq_linear_choice(
+            M, N, K, rfq.RFQ_FMT_BF16 if hif4 else rfq.RFQ_FMT_MXFP4, not no_res, amax_phi,
+            fused)["kernel"] == rfq.RFQ_KERNEL_CLUSTER:
+        t_kernel = "gemm_small_kernel"
     if hif4:
         aq_bytes = _act_quant_bytes(Mb, K, "hif4", not no_res, operand=not quant_only)
         aq_kernel = "act_quant_hif4_amax_kernel" if amax_fused else "act_quant_hif4_kernel"
