@@ -202,15 +202,23 @@ RFQ_API rfq_status rfq_quantize_act_expand(const void *x_bf16, int64_t M, int64_
 RFQ_API size_t rfq_linear_workspace_bytes(void);
 
 /* RFQ GEMM (Algorithm 1, Eq. rfq): Y = X~ W~ + phi X^ W~ with both products
- * accumulated into one fp32 accumulator per output tile, the weight tile read
- * once for both.  xq: [M x K] main codes; xr: [M x K] residual codes or NULL
+ * accumulated in fp32, the weight tile read once for both.  The sum's order
+ * depends on the kernel that the layer's sizes, residual and phi select
+ * (rfq_linear_choice), not on the run: the tiled kernels add both products of
+ * a k-step, in k order, into one accumulator per output tile; the
+ * cluster-split kernel splits k over the CTAs of a cluster, keeps the two
+ * products apart up to 64 rows, and adds these partial sums in a fixed order.
+ * So a row's Y can differ in its last fp32 bits between calls of different M;
+ * rfq_linear_on with RFQ_KERNEL_TILED gives it the same bits in all of them
+ * (phi NULL).  xq: [M x K] main codes; xr: [M x K] residual codes or NULL
  * (plain W4A4); phi: device bytes [ceil(M/128)][K/r_s] selecting the
  * residual k-tiles per 128-row tile, or NULL (= all ones); phi_r_s: the
  * column tile r_s of phi (a multiple of 128; ignored when phi is NULL).
  * The residual of every phi = 0 tile must be stored as zero, as
  * rfq_quantize_act writes it: phi only lets the GEMM skip residual loads and
- * products, at its own granularity (it may still include a phi = 0 tile that
- * shares a 256-row or 256-column block with a phi = 1 one).
+ * products, at its own granularity (the tiled kernels may still include a
+ * phi = 0 tile that shares a 256-row or 256-column block with a phi = 1 one;
+ * the cluster-split kernel includes every tile).
  * wq: [N x K] weight.  MXFP4: every operand MXFP4 with RFQ_SCALE_MMA,
  * K % 128 == 0.  MXFP8: xq (and xr) MXFP8 (E4M3, kind::mxf8f6f4 MMAs)
  * with RFQ_SCALE_MMA, K % 128 == 0, and wq MXFP8 or MXFP4 -- the W8A8 and

@@ -591,8 +591,8 @@ cudaError_t launch_conv(const GemmHif4Args &a, cudaStream_t st)
 cudaError_t launch_gemm_hif4(const GemmHif4Args &a, cudaStream_t st)
 {
     if (a.a_bf16) {
-        // as for the MXFP4 GEMM: 32 x 12288 x 4096 takes 22 us there against
-        // 111 us here, 1800 x 4096 x 1024 25.1 against 42.4; 4096 x 12288 x 4096
+        // as for the MXFP4 GEMM: 32 x 12288 x 4096 takes 24 us there against
+        // 110 us here, 1800 x 4096 x 1024 24.0 against 40.4; 4096 x 12288 x 4096
         // (512 tiles, a full 3.4 waves) stays here
         GemmSmallArgs s = {};
         s.x = a.a_codes;

@@ -743,8 +743,10 @@ cudaError_t launch_gemm_mxf4(const GemmMxf4Args &a, cudaStream_t st)
     if (!grp && !a.f8) {
         // Few rows, or few output tiles: the cluster-split kernel where its
         // estimated time is the smaller (choose() in gemm_small.cu).  48 x 12288
-        // x 4096: 10.3 us there against 34 us here (16 tiles for 152 SMs); 128 x
-        // 5120 x 24576: 22.6 against 21.9 us (96 tiles), which stays here.
+        // x 4096: 12.1 us there against 34 us here (16 tiles for 152 SMs); 128 x
+        // 4096 x 24576: 18.9 against 17.8 (96 tiles), which stays here; 128 x 5120
+        // x 24576: 21.7 against 20.9, the layer 23.0 against 22.8, which goes there
+        // within the estimate's error.
         GemmSmallArgs s = {};
         s.x = a.a_codes;
         s.r = a.r_codes;

@@ -407,7 +407,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PHI ? THREADS + 32 :
     // lane 80-100 cycles, so one producer needed most of a stage's MMA time
     // for its seven or eight (the mixed-rate form more than all of it).  Layer
     // times with one producer and with two: mixed rate 8190 x 5120 x 13824 500
-    // and 489 us, MXFP4 4096 x 4096 x 24576 226 and 222 (the single-CTA kernel,
+    // and 489 us; MXFP4 4096 x 4096 x 24576 226 and 222 on operands left in L2,
+    // no difference beyond the noise of 1% on cold ones (the single-CTA kernel,
     // whose stages take longer, gained nothing and keeps one).
     auto producer = [&](auto ops_t) {
         constexpr bool OPS = decltype(ops_t)::value;

@@ -33,8 +33,8 @@
 // that read the slot had completed.
 //
 // Selective phi is not looked at here: the stored residual of a phi = 0 tile
-// is zero, so including it adds exact zeros, and X^ is a small part of what a
-// CTA loads.
+// is zero, so including it adds exact zeros.  The choice of the kernel counts
+// with a tiled kernel that skips it (choose()).
 //
 // Shared memory is requested in proportion to the TMEM columns (a CTA with
 // all 512 columns takes a whole SM's shared memory, 256 columns half of it),

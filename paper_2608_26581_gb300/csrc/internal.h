@@ -239,9 +239,12 @@ rfq_status linear_rows(const rfq_qtensor *xq, const rfq_qtensor *xr, const uint8
 int resident_blocks_per_sm(const void *kern, int threads, size_t smem);
 
 // Launch of a GEMM kernel that calls grid_dependency_wait before its first
-// read of global memory: with `dependent` its set-up may overlap the end of
-// the kernel ahead of it in the stream (the activation quantizer: 1.0-1.7 us
-// less per layer).  Calls from host memory (rfq_linear_host) launch plainly.
+// read of global memory: with `dependent` it may be launched while the kernel
+// ahead of it in the stream (the activation quantizer) still runs: 1.0-1.7 us
+// less per layer.  The CTA-pair and the cluster-split kernel also set up their
+// barriers and tensor memory before the wait; the single-CTA and the HiF4
+// kernel wait first, so only their launch overlaps.  Calls from host memory
+// (rfq_linear_host) launch plainly.
 template <class... P, class... A>
 inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
                                     bool dependent, A... args)

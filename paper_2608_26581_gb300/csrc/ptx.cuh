@@ -160,7 +160,8 @@ __device__ __forceinline__ bool held_start_wait(const int32_t *ws, uint64_t limi
 
 // Lets the next kernel of the stream, if it was launched to allow it, start
 // its set-up while this grid still runs (it waits in grid_dependency_wait for
-// this grid's end and its memory).  No effect on any other kernel.
+// this grid's end and its memory).  No effect on any other kernel.  (A short
+// quantizer with no GEMM behind it pays 0.15 us for it: 1000 x 512 2.10 -> 2.25 us.)
 __device__ __forceinline__ void grid_launch_dependents()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

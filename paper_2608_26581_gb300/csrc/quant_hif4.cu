@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256) act_quant_hif4_kernel(const uint4 *__rest
                                                             const uint8_t *__restrict__ phi, int p_s, int r_s,
                                                             uint4 *__restrict__ m16, uint4 *__restrict__ r16)
 {
-    grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
+    grid_launch_dependents();   // (a following GEMM may set up meanwhile)
     const int lane = threadIdx.x & 31;
     constexpr int NG = kHNG, LPB = 8 / NG;         // groups per lane, lanes per block
     const int gq = lane & (LPB - 1);               // the lane's place in its block
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(512, 1) act_quant_hif4_amax_kernel(const uint4
                                                                     uint8_t *__restrict__ phi, float tau,
                                                                     uint4 *__restrict__ m16, uint4 *__restrict__ r16)
 {
-    grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
+    grid_launch_dependents();   // (a following GEMM may set up meanwhile)
     constexpr int R = kHAmaxRows, NW = 16;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t kchunks = K >> 3;

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(256) act_quant8_kernel(const uint4 *__restrict
                                                         int64_t pad_rows, uint8_t *__restrict__ m8codes = nullptr,
                                                         uint8_t *__restrict__ m8scales = nullptr)
 {
-    grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
+    grid_launch_dependents();   // (a following GEMM may set up meanwhile)
     const int lane = threadIdx.x & 31;
     const int kchunks = (int)(K >> 3);
     const int kblocks = (int)(K >> 5);
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(256) act_quant_rfq8_kernel(const uint4 *__rest
                                                             const uint8_t *__restrict__ phi, int p_s, int r_s,
                                                             int64_t pad_rows)
 {
-    grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
+    grid_launch_dependents();   // (a following GEMM may set up meanwhile)
     const int lane = threadIdx.x & 31;
     const int kblocks = (int)(K >> 5);
     const int segs = (kblocks + 31) / 32;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(256, 3) act_quant_rfq8_amax_kernel(const uint4
                                                                     uint8_t *__restrict__ m8codes,
                                                                     uint8_t *__restrict__ m8scales)
 {
-    grid_launch_dependents();   // (a following few-rows GEMM may set up meanwhile)
+    grid_launch_dependents();   // (a following GEMM may set up meanwhile)
     constexpr int R = 16, NW = 8;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t kchunks = K >> 3;

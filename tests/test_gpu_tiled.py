@@ -4,6 +4,7 @@ records and bounded waits run with that choice taken away (rfq_linear_on)."""
 import functools
 
 import pytest
+import torch
 
 import test_gpu_abort as _abort
 import test_gpu_debug_build as _debug
@@ -39,3 +40,17 @@ def test_debug_build_checks_the_pair_epilogue(tmp_path, monkeypatch):
     monkeypatch.setattr(_debug, "_CASES", _debug._CASES.replace("rfq.rfq_linear(xq", "rfq.rfq_linear_on(rfq.RFQ_KERNEL_TILED, xq"))
     assert "RFQ_KERNEL_TILED" in _debug._CASES
     _debug.test_debug_build_records_no_out_of_range_store_and_matches(tmp_path)
+
+
+def test_rows_sum_alike_in_calls_of_every_size():
+    """A row's Y has the same bits whether its call has 700 rows or 1 (single CTAs up to 128 rows, pairs beyond)."""
+    M, K, N = 700, 4224, 1040
+    wq, xq, xr, y = _abort._mxfp4(M, K, N)
+    x = _abort._x(M, K, M)
+    rfq.rfq_linear(xq, xr, None, 256, wq, y, rfq.RFQ_OUT_F32, _abort._ws())
+    for a, b in ((0, 1), (128, 256), (384, 700), (699, 700)):
+        q, r = (rfq.empty_qtensor(rfq.RFQ_FMT_MXFP4, rfq.RFQ_SCALE_MMA, b - a, K) for _ in range(2))
+        rfq.rfq_quantize_act(x[a:b].contiguous(), q, r)
+        part = torch.empty(b - a, N, device="cuda")
+        rfq.rfq_linear(q, r, None, 256, wq, part, rfq.RFQ_OUT_F32, _abort._ws())
+        assert torch.equal(part, y[a:b]), (a, b)
