@@ -915,7 +915,7 @@ float tiled_us(const GemmSmallArgs &a, int64_t rows)
 // tiled kernels skip what is not there, and need a quarter less.  A layer
 // without a residual, or with phi (of which nothing is known here, so with no
 // tile kept, the tiled kernels' best), therefore has to pass a second
-// comparison, of estimates fitted to 2,144 layers of this kind timed on both
+// comparison, of estimates fitted to 2,144 layers that were timed on both
 // kernels, M 1-4096, K 512-13824, N 512-24576 (relative error 5%; bf16 7%):
 //   here   one + cluster cs + wave waves + kb (100 KB copied per SM, in turn) +
 //          hbm (MB of W~) + epi (10,000 outputs of a CTA, in turn) + moved (MB
